@@ -95,20 +95,22 @@ F3DC_DEV bool mbar_try_wait_sleep(uint64_t *bar, uint32_t parity, uint32_t hint_
 
 // Waits for the phase with the given parity to complete.  Gives up (returns
 // false) when *abort is set by another thread or after kWaitLimitNs; in the
-// latter case it sets *abort and records kDevTimeout.
+// latter case it sets *abort and records kDevTimeout.  The code is kept short:
+// it is inlined at every wait of kernels whose warps share an instruction cache.
 F3DC_DEV bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort, uint32_t *err)
 {
     if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer();
-    while (true) {
-        if (mbar_try_wait_sleep(bar, parity, 100000u)) return true;
+    const uint64_t end = globaltimer() + kWaitLimitNs;
+#pragma unroll 1
+    while (!mbar_try_wait_sleep(bar, parity, 100000u)) {
         if (*abort) return false;
-        if (globaltimer() - t0 > kWaitLimitNs) {
+        if (globaltimer() > end) {
             *abort = 1;
             raise_error(err, kDevTimeout);
             return false;
         }
     }
+    return true;
 }
 
 // Spins (bounded) for ns nanoseconds; used to let in-flight TMA copies land
@@ -180,6 +182,19 @@ F3DC_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "
 // the next kernel be scheduled early; its CTAs still wait in griddep_wait().
 F3DC_DEV void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 F3DC_DEV void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Register split between warpgroups (every warp of a warpgroup executes the
+// same one).  The sum over the block must not exceed its registers at launch.
+template <int N>
+F3DC_DEV void reg_inc()
+{
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+F3DC_DEV void reg_dec()
+{
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
 
 // Orders this thread's generic-proxy shared-memory writes before later
 // async-proxy (tensor core / TMA) reads of the same memory.
@@ -267,6 +282,15 @@ F3DC_DEV void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;
 // every lane's outcome, so a warp takes the same branch around its
 // warp-collective instructions even when a bounded wait gives up in one lane
 F3DC_DEV bool warp_all(bool v) { return __all_sync(0xffffffffu, v); }
+
+// mbar_wait by a whole warp: true in every lane, or false in every lane.  The
+// vote on the first look comes before any branch, so a wait that is already
+// over costs one look, one vote and no divergence.
+F3DC_DEV bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort, uint32_t *err)
+{
+    if (warp_all(mbar_try_wait(bar, parity))) return true;
+    return warp_all(mbar_wait(bar, parity, abort, err));
+}
 
 // D[tmem] (+)= A[smem desc] * B[smem desc]^T, bf16 inputs, fp32 accumulate.
 F3DC_DEV void mma_bf16_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)

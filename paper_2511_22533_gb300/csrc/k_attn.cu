@@ -6,31 +6,45 @@
 //           tokens (Supp. Sec. F cross-attention)
 //   mode 2  one sequence (diagnostic entry point)
 //
-// Persistent kernel, one CTA per SM (320 threads).  A work item is two
+// Persistent kernel, one CTA per SM (384 threads).  A work item is two
 // 128-query tiles A and B of one head that share their keys: the K / V tiles
 // are loaded once for both, and the two tiles' score / softmax / P V chains
 // run side by side, so while one tile's softmax works the tensor core serves
 // the other's MMAs.
 //   warp 0     TMA producer: the item's two Q tiles (double-buffered across
 //              items), K / V tiles of 128 keys into a 4-deep ring
-//   warp 1     TMEM allocator + tcgen05.mma issuer (the whole warp runs the
-//              loop and votes on every barrier outcome; elect.sync issues).
-//              Per key tile j:  S_A(j), S_B(j)   (S_t = Q_t K_j^T, N=128,
-//              K=dh; each once the softmax has loaded the previous S_t),
-//              then P_A V(j-1), P_B V(j-1)        (O_t += P_t V, N=dh, K=128,
-//              each once P_t is written; P read straight from TMEM)
-//   warps 2-5  softmax of tile A, warps 6-9 of tile B: one thread per query
-//              row (TMEM lane = row), all 128 keys of each key tile, online
-//              softmax with the row's running max m and sum l, in one pass
-//              over the key tile's two halves of 64 keys: each half is
-//              loaded once, its maximum raises the reference max m only when
-//              it exceeds m by more than 2^8 (O_t, l rescaled in place; a
-//              raise in the second half recomputes the first half's P), and
-//              P = exp2(S scale - m) goes to TMEM P_t as bf16 pairs (once
-//              P V of the previous key tile has read P_t).  The S buffer is
-//              released for the next key tile's MMA as soon as its last load
-//              landed.  O_t stays in TMEM for the whole item; at the item's
-//              end O_t / l is stored as bf16.
+//   warps 1, 2 tcgen05.mma issuers of tile A and of tile B (the whole warp
+//              runs the loop and votes on every barrier outcome; elect.sync
+//              issues), so neither tile's chain waits behind the other's.
+//              Per key tile g: S_t(g + 1) = Q_t K^T (N=128, K=dh; once the
+//              softmax has loaded S_t(g); also across items), then
+//              O_t += P_t V(g) (N=dh, K=128; once P_t is written; P read
+//              straight from TMEM).  Warp 1 allocates TMEM.
+//   warp 3     idle (completes the warpgroup whose registers are given away)
+//   warps 4-7  softmax of tile A, warps 8-11 of tile B: one thread per query
+//              row (TMEM lane = row).  The row's 128 scores of a key tile
+//              are loaded into registers at once and S_t is released for
+//              the next key tile's MMA; P = exp2(S scale - m) goes to TMEM
+//              P_t as bf16 pairs; l sums P in fp32.  O_t stays in TMEM for
+//              the whole item; at its end O_t / l is stored as bf16.
+// The reference m is the row's maximum over the item's first key tile (and
+// the ragged last one, if it is 2^8 above).  A later score above m is no
+// loss: P, l and O are floating point, with the same 8 exponent bits, so only
+// an overflow would be, and that is seen at the item's end (l above 2^64, O
+// not finite).  The CTA then does its items a second time with the maximum of
+// every key tile, m raised (O_t and l rescaled in place) when a tile's maximum
+// is 2^8 above it.  So the loop over the key tiles takes no maximum and has
+// no branch on the data.
+// What bounds it: the softmax warps.  Per key tile of 128 x 128 scores an SM's
+// exponent unit needs 512 clocks (32 per clock) and the tensor core 512; the
+// kernel takes ~990 (4096 x 4096 x 16 heads, dh 64: 66.2 us = 1038 TFLOP/s;
+// before -- one issuer warp, a maximum of every half tile, ~1250 clocks --
+// 79.1 us; 1229 x 1374: 17.6 -> 15.9 us).  A softmax warp alone needs ~730
+// clocks per tile (load, exponents, store), and the two of an SM sub-partition
+// mostly compete for the exponent unit at the same time.  Measured slower: 16
+// softmax warps with half a row each (73 us: the waits' instructions double),
+// turn-taking of the two warps through mbarriers, loading the next tile's
+// scores under this one's exponents.
 // TMEM: S_A S_B (fp32, 128 columns each) | O_A O_B (dh each) | P_A P_B (64).
 // V is the MN-major B operand of the P V MMA straight from its row-major
 // TMA tile.  Keys beyond a sample's count are masked to -inf before the
@@ -44,8 +58,12 @@ namespace f3dc {
 
 namespace {
 
-constexpr int kAttnThreads = 320;  // producer, MMA issuer, 2 x 4 softmax warps
+constexpr int kAttnThreads = 384;  // producer, MMA issuer, two idle warps, 2 x 4 softmax warps
 constexpr int kKVStages = 4;
+// Registers per thread after the split.  The launch has 384 x 168 = 64512; a
+// softmax thread holds a whole score row of a key tile (128 floats).
+constexpr int kCtrlRegs = 72, kSoftmaxRegs = 216;
+static_assert(128 * kCtrlRegs + 256 * kSoftmaxRegs <= 384 * 168, "register split above the launch's total");
 
 template <int DH>
 struct AttnCfg {
@@ -152,18 +170,19 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     uint64_t *drain = o_free + 2;
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
+    volatile int *redo_flag = abort_flag + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     griddep_launch();
 
     if (threadIdx.x == 0) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&q_full[b], 1);
-            mbar_init(&q_empty[b], 1);
+            mbar_init(&q_empty[b], 2);  // both MMA warps
         }
         for (int s = 0; s < kKVStages; ++s) {
             mbar_init(&kv_full[s], 1);
-            mbar_init(&kv_empty[s], 1);
+            mbar_init(&kv_empty[s], 2);
         }
         for (int t = 0; t < 2; ++t) {
             mbar_init(&s_full[t], 1);
@@ -172,8 +191,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             mbar_init(&pv_done[t], 1);
             mbar_init(&o_free[t], 4);
         }
-        mbar_init(drain, 1);
+        mbar_init(drain, 2);
         *abort_flag = 0;
+        *redo_flag = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -192,54 +212,73 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_holder;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
     // the previous kernel's outputs (Q / K / V, the row plan) are complete
     griddep_wait();
-    const int n_tiles = p.n_tiles_dev ? *p.n_tiles_dev : p.n_tiles;
+    const int n_tiles = __shfl_sync(0xffffffffu, p.n_tiles_dev ? *p.n_tiles_dev : p.n_tiles, 0);
     const int total = total_items(p, n_tiles);
+
+    // Every warp ends a pass over the CTA's items here, also when the kernel is
+    // aborting (each role's waits are bounded); a second pass follows if the
+    // softmax asked for one.
+    auto again = [&]() {
+        asm volatile("bar.sync 1, %0;" ::"n"(kAttnThreads) : "memory");
+        return *redo_flag != 0 && *abort_flag == 0;
+    };
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
-            tma_prefetch(&tmq);
-            tma_prefetch(&tmk);
-            tma_prefetch(&tmv);
-            uint32_t kv_it = 0, item_it = 0;
-            bool ok = true;
-            for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-                Item it;
-                if (!decode_item(p, w, n_tiles, it)) continue;
-                const uint32_t my_it = item_it++;
-                // Q buffer qb holds items qb, qb + 2, ...: its (my_it / 2)-th use
-                const uint32_t qb = my_it & 1, qph = (my_it >> 1) & 1;
-                if (!mbar_wait(&q_empty[qb], qph ^ 1, abort_flag, p.err)) break;
-                mbar_arrive_expect_tx(&q_full[qb], 2 * Cfg::kTileBytes);
-                for (int t = 0; t < 2; ++t)
-                    tma_load_2d(sQ + (2 * qb + t) * Cfg::kTileBytes, &tmq, p.q_col0 + it.h * DH, it.q_row0 + 128 * t,
-                                &q_full[qb]);
-                const int nkt = (it.nk + 127) / 128;
-                for (int j = 0; j < nkt; ++j, ++kv_it) {
-                    const int s = kv_it % kKVStages;
-                    const uint32_t ph = (kv_it / kKVStages) & 1;
-                    if (!mbar_wait(&kv_empty[s], ph ^ 1, abort_flag, p.err)) {
-                        ok = false;
-                        break;
+        reg_dec<kCtrlRegs>();
+        uint32_t kv_it = 0, item_it = 0;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            if (lane == 0) {
+                if (pass == 0) {
+                    tma_prefetch(&tmq);
+                    tma_prefetch(&tmk);
+                    tma_prefetch(&tmv);
+                }
+                bool ok = true;
+#pragma unroll 1
+                for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+                    Item it;
+                    if (!decode_item(p, w, n_tiles, it)) continue;
+                    const uint32_t my_it = item_it++;
+                    // Q buffer qb holds items qb, qb + 2, ...: its (my_it / 2)-th use
+                    const uint32_t qb = my_it & 1, qph = (my_it >> 1) & 1;
+                    if (!mbar_wait(&q_empty[qb], qph ^ 1, abort_flag, p.err)) break;
+                    mbar_arrive_expect_tx(&q_full[qb], 2 * Cfg::kTileBytes);
+                    for (int t = 0; t < 2; ++t)
+                        tma_load_2d(sQ + (2 * qb + t) * Cfg::kTileBytes, &tmq, p.q_col0 + it.h * DH,
+                                    it.q_row0 + 128 * t, &q_full[qb]);
+                    const int nkt = (it.nk + 127) / 128;
+#pragma unroll 1
+                    for (int j = 0; j < nkt; ++j, ++kv_it) {
+                        const int s = kv_it % kKVStages;
+                        const uint32_t ph = (kv_it / kKVStages) & 1;
+                        if (!mbar_wait(&kv_empty[s], ph ^ 1, abort_flag, p.err)) {
+                            ok = false;
+                            break;
+                        }
+                        // fault injection (tests of the failure path): the last
+                        // key tile of CTA 0's first item is never loaded, so the
+                        // waits on it (and on what follows it) run out while the
+                        // earlier tiles went through, and the kernel aborts
+                        if (p.fault_skip_kv && blockIdx.x == 0 && my_it == 0 && j == nkt - 1) continue;
+                        mbar_arrive_expect_tx(&kv_full[s], 2 * Cfg::kTileBytes);
+                        tma_load_2d(sK + s * Cfg::kTileBytes, &tmk, p.k_col0 + it.h * DH, it.kv_row0 + j * 128,
+                                    &kv_full[s]);
+                        tma_load_2d(sV + s * Cfg::kTileBytes, &tmv, p.v_col0 + it.h * DH, it.kv_row0 + j * 128,
+                                    &kv_full[s]);
                     }
-                    // fault injection (tests of the failure path): the last
-                    // key tile of CTA 0's first item is never loaded, so the
-                    // waits on it (and on what follows it) run out while the
-                    // earlier tiles went through, and the kernel aborts
-                    if (p.fault_skip_kv && blockIdx.x == 0 && my_it == 0 && j == nkt - 1) continue;
-                    mbar_arrive_expect_tx(&kv_full[s], 2 * Cfg::kTileBytes);
-                    tma_load_2d(sK + s * Cfg::kTileBytes, &tmk, p.k_col0 + it.h * DH, it.kv_row0 + j * 128,
-                                &kv_full[s]);
-                    tma_load_2d(sV + s * Cfg::kTileBytes, &tmv, p.v_col0 + it.h * DH, it.kv_row0 + j * 128,
-                                &kv_full[s]);
                 }
             }
+            __syncwarp();
+            if (!again()) break;
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer
+    } else if (warp <= 2) {
+        // ------------------------------------------------ MMA issuer of one query tile
+        reg_dec<kCtrlRegs>();
         // Every lane runs the loop (a converged warp keeps the descriptors
         // warp-uniform) and takes each barrier outcome as a warp vote;
         // elect.sync issues.  Key tile g (counted over the CTA's whole run)
@@ -251,271 +290,262 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // descriptors of the stage bases; a K step of 16 elements inside a
             // 128B / 64B swizzle atom advances the start address by 32 bytes,
             // i.e. the descriptor by 2
-            const uint64_t q_desc0 = make_sdesc(smem_u32(sQ), 16, Cfg::kAtom, Cfg::kSwz);
+            const int t = warp - 1;
+            const uint64_t q_desc0 = make_sdesc(smem_u32(sQ + t * Cfg::kTileBytes), 16, Cfg::kAtom, Cfg::kSwz);
             const uint64_t k_desc0 = make_sdesc(smem_u32(sK), 16, Cfg::kAtom, Cfg::kSwz);
             const uint64_t v_desc0 = make_sdesc(smem_u32(sV), Cfg::kAtom, Cfg::kAtom, Cfg::kSwz);
             constexpr uint64_t kStageStep = Cfg::kTileBytes >> 4, kVRowStep = (16 * Cfg::kRowBytes) >> 4;
-            auto wait = [&](uint64_t *bar, uint32_t ph) { return warp_all(mbar_wait(bar, ph, abort_flag, p.err)); };
-            uint32_t g = 0, item_it = 0;
-            bool ok = true;
-            for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-                Item it;
-                if (!decode_item(p, w, n_tiles, it)) continue;
-                const uint32_t my_it = item_it++;
-                const uint32_t nkt = (uint32_t)((it.nk + 127) / 128);
-                const uint32_t qb = my_it & 1;
-                if (!wait(&q_full[qb], (my_it >> 1) & 1)) break;
-                // step j: S of key tile j (j < nkt), then P V of key tile j - 1
-                // (j >= 1); every item has at least one key tile (a sample
-                // without active tokens owns no query tile, and the entry
-                // points reject nk < 1)
-                for (uint32_t j = 0; j <= nkt && ok; ++j) {
-                    if (j < nkt) {
-                        // S_A and S_B of key tile gt, each once the softmax
-                        // has read the previous S of its tile
-                        const uint32_t gt = g + j;
-                        if (!wait(&kv_full[gt % kKVStages], (gt / kKVStages) & 1)) {
-                            ok = false;
-                            break;
+            auto wait = [&](uint64_t *bar, uint32_t ph) { return warp_wait(bar, ph, abort_flag, p.err); };
+            // One loop, S one key tile ahead of P V (also across items), so
+            // that each is in the code once: the instruction cache is what
+            // ten warps at different places of a long kernel share.
+            uint32_t g = 0, item = 0;  // S: key tile g of the CTA's run, in its item number item
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                int w = (int)blockIdx.x - (int)gridDim.x;
+                uint32_t nkt = 0, j = 0;                // key tiles of the item, S's within it
+                bool pending = false, p_first = false;  // P V of key tile g - 1, the first of its item
+                uint32_t p_par = 0;                     // o_free's phase for that item
+#pragma unroll 1
+                while (true) {
+                    if (j == nkt) {  // the next real work item
+                        if (nkt) ++item;
+                        nkt = j = 0;
+#pragma unroll 1
+                        while (nkt == 0 && (w += gridDim.x) < total) {
+                            Item it;
+                            const uint32_t n = decode_item(p, w, n_tiles, it) ? (uint32_t)((it.nk + 127) / 128) : 0u;
+                            nkt = __shfl_sync(0xffffffffu, n, 0);
                         }
-                        const uint64_t kd = k_desc0 + (gt % kKVStages) * kStageStep;
-                        for (int t = 0; t < 2; ++t) {
-                            if (!wait(&s_free[t], (gt & 1) ^ 1)) {
-                                ok = false;
-                                break;
-                            }
-                            tc_fence_after();
-                            const uint64_t qd = q_desc0 + (uint64_t)(2 * qb + t) * kStageStep;
-#pragma unroll
-                            for (int kk = 0; kk < DH / 16; ++kk)
-                                mma_bf16_elect(tmem + t * 128, qd + 2 * kk, kd + 2 * kk, idesc_s, kk > 0);
-                            mma_commit_elect(&s_full[t]);
-                        }
-                        if (!ok) break;
-                        if (j + 1 == nkt) mma_commit_elect(&q_empty[qb]);  // every S of the item issued
                     }
-                    if (j >= 1) {
-                        // P_t V of key tile gp, once P_t is written
-                        const uint32_t gp = g + j - 1;
-                        const bool fresh = j == 1;
-                        const uint64_t vd = v_desc0 + (gp % kKVStages) * kStageStep;
-                        for (int t = 0; t < 2; ++t) {
-                            // the item's first P V overwrites O_t: the softmax
-                            // must have read the previous item's
-                            if (fresh && !wait(&o_free[t], (my_it & 1) ^ 1)) {
-                                ok = false;
-                                break;
-                            }
-                            if (!wait(&p_full[t], gp & 1)) {
-                                ok = false;
-                                break;
-                            }
-                            tc_fence_after();
+                    if (nkt) {
+                        // S_t, once the softmax has loaded the previous S_t
+                        const uint32_t st = g % kKVStages, qb = item & 1;
+                        if (j == 0 && !wait(&q_full[qb], (item >> 1) & 1)) break;
+                        if (!wait(&kv_full[st], (g / kKVStages) & 1)) break;
+                        if (!wait(&s_free[t], (g & 1) ^ 1)) break;
+                        tc_fence_after();
+                        const uint64_t kd = k_desc0 + st * kStageStep, qd = q_desc0 + (uint64_t)(2 * qb) * kStageStep;
 #pragma unroll
-                            for (int kk = 0; kk < 8; ++kk)
-                                mma_bf16_ts_elect(tmem + Cfg::kColO + t * DH, tmem + Cfg::kColP + t * 64 + kk * 8,
-                                                  vd + kk * kVRowStep, idesc_o, !(fresh && kk == 0));
-                            mma_commit_elect(&pv_done[t]);
-                        }
-                        if (!ok) break;
-                        mma_commit_elect(&kv_empty[gp % kKVStages]);  // both tiles' S and P V of the stage issued
+                        for (int kk = 0; kk < DH / 16; ++kk)
+                            mma_bf16_elect(tmem + t * 128, qd + 2 * kk, kd + 2 * kk, idesc_s, kk > 0);
+                        mma_commit_elect(&s_full[t]);
+                        if (j + 1 == nkt) mma_commit_elect(&q_empty[qb]);  // every S_t of the item issued
                     }
+                    if (pending) {
+                        // P_t V, once P_t is written; the item's first overwrites
+                        // O_t, which the softmax must have read for the previous item
+                        const uint32_t gp = g - 1, st = gp % kKVStages;
+                        if (p_first && !wait(&o_free[t], p_par)) break;
+                        if (!wait(&p_full[t], gp & 1)) break;
+                        tc_fence_after();
+                        const uint64_t vd = v_desc0 + st * kStageStep;
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk)
+                            mma_bf16_ts_elect(tmem + Cfg::kColO + t * DH, tmem + Cfg::kColP + t * 64 + kk * 8,
+                                              vd + kk * kVRowStep, idesc_o, kk > 0 || !p_first);
+                        mma_commit_elect(&pv_done[t]);
+                        mma_commit_elect(&kv_empty[st]);
+                    }
+                    if (!nkt) break;
+                    pending = true;
+                    p_first = j == 0;
+                    p_par = (item & 1) ^ 1;
+                    ++j;
+                    ++g;
                 }
-                g += nkt;
+                if (!again()) break;
             }
         }
+    } else if (warp < 4) {
+        reg_dec<kCtrlRegs>();  // idle: gives its registers to the softmax warps
+        if (again()) again();
     } else {
         // ------------------------------------------------ softmax warps
+        reg_inc<kSoftmaxRegs>();
         const int q = warp & 3;              // TMEM lane quarter of this warp
-        const int t = (warp - 2) >> 2;       // query tile: warps 2-5 A, 6-9 B
+        const int t = (warp - 4) >> 2;       // query tile: warps 4-7 A, 8-11 B
         const int row = q * 32 + lane;
         const uint32_t tl = (uint32_t)(q * 32) << 16;
         const uint32_t s_addr = tmem + tl + t * 128;
         const uint32_t o_addr = tmem + tl + Cfg::kColO + t * DH;
         const uint32_t p_addr = tmem + tl + Cfg::kColP + t * 64;
-        auto wait = [&](uint64_t *bar, uint32_t ph) { return warp_all(mbar_wait(bar, ph, abort_flag, p.err)); };
+        auto wait = [&](uint64_t *bar, uint32_t ph) { return warp_wait(bar, ph, abort_flag, p.err); };
         // S_t of key tile g completes s_full[t] (phase g), the four warps'
         // arrivals on s_free[t] / p_full[t] complete phase g once S_t is
         // loaded / P_t written, and P_t V of tile g completes pv_done[t]; a
         // wait that gives up (the kernel is aborting) ends this warp's loop
-        uint32_t g = 0;  // key tiles of this CTA's earlier items
-        for (int w = blockIdx.x; w < total; w += gridDim.x) {
-            Item it;
-            if (!decode_item(p, w, n_tiles, it)) continue;
-            const int nkt = (it.nk + 127) / 128;
-            float m_ref = -INFINITY, l_run = 0.f;
-            bool ok = true;
-            for (int j = 0; j < nkt; ++j) {
-                const uint32_t gt = g + (uint32_t)j;
-                if (!wait(&s_full[t], gt & 1)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                // one pass over the tile's two halves of 64 keys: load, take the
-                // half's maximum, raise the reference max when it grew by more
-                // than 2^8 (warp-uniform), then exponents against it.  A raise
-                // in the second half makes the first half's P stale: its S is
-                // still in TMEM (released only after this check), so it is
-                // recomputed against the new max.
-                const int valid = it.nk - j * 128;  // < 128 only on the last, ragged key tile
-                f32x2 sum0 = {0.f, 0.f}, sum1 = {0.f, 0.f};
-                bool pv_ready = gt == 0;  // P V of the previous key tile done (P_t, O_t free)
-                bool o_live = j > 0;      // O_t holds this item's earlier tiles
-                auto ensure_pv = [&]() {
-                    if (!pv_ready) {
-                        pv_ready = wait(&pv_done[t], (gt - 1) & 1);
-                        if (!pv_ready) ok = false;
-                    }
-                    return pv_ready;
-                };
-                auto rescale = [&](float alpha) {
-                    if (o_live) {
-                        tc_fence_after();
-#pragma unroll
-                        for (int d0 = 0; d0 < DH; d0 += 16) {
-                            uint32_t r[16];
-                            tmem_ld16(o_addr + d0, r);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int d = 0; d < 16; ++d) r[d] = __float_as_uint(__uint_as_float(r[d]) * alpha);
-                            tmem_st16(o_addr + d0, r);
-                        }
-                    }
-                    l_run *= alpha;
-                };
-                // exponents of one half against m_ref, P to TMEM as bf16 pairs
-                auto emit_half = [&](int hb, const float (&sv)[64]) {
-                    const float m_use = m_ref == -INFINITY ? 0.f : m_ref;
-                    const f32x2 sc2 = {p.scale_log2, p.scale_log2}, nm2 = {-m_use, -m_use};
-                    f32x2 s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
-                    uint32_t pw[32];
-#pragma unroll
-                    for (int c = 0; c < 32; c += 2) {
-                        const int k0 = 2 * c;
-                        const f32x2 x0 = ffma2({sv[k0], sv[k0 + 1]}, sc2, nm2);
-                        const f32x2 x1 = ffma2({sv[k0 + 2], sv[k0 + 3]}, sc2, nm2);
-                        const f32x2 e0 = {exp2_fast(x0.x), exp2_fast(x0.y)};
-                        const f32x2 e1 = {exp2_fast(x1.x), exp2_fast(x1.y)};
-                        s0 = fadd2(s0, e0);
-                        s1 = fadd2(s1, e1);
-                        pw[c] = pack_bf16x2(e0.x, e0.y);
-                        pw[c + 1] = pack_bf16x2(e1.x, e1.y);
-                    }
-                    if (!ensure_pv()) return;
-                    tmem_st32(p_addr + 32 * hb, pw);
-                    if (hb == 0) {
-                        sum0 = s0;
-                        sum1 = s1;
-                    } else {
-                        sum0 = fadd2(sum0, s0);
-                        sum1 = fadd2(sum1, s1);
-                    }
-                };
-                auto load_half = [&](int hb, float (&sv)[64]) {
-                    uint32_t r0[32], r1[32];
-                    tmem_ld32(s_addr + 64 * hb, r0);
-                    tmem_ld32(s_addr + 64 * hb + 32, r1);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        sv[c] = __uint_as_float(r0[c]);
-                        sv[32 + c] = __uint_as_float(r1[c]);
-                    }
-                    if (valid < 128) {
-#pragma unroll
-                        for (int c = 0; c < 64; ++c)
-                            if (64 * hb + c >= valid) sv[c] = -INFINITY;
-                    }
-                };
-                auto half_max = [&](const float (&sv)[64]) {
-                    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int c = 0; c < 64; c += 8) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) mx4[e] = fmax3(mx4[e], sv[c + e], sv[c + 4 + e]);
-                    }
-                    return fmax3(mx4[0], mx4[1], fmaxf(mx4[2], mx4[3])) * p.scale_log2;
-                };
-                // raise m_ref to cover mx when it grew by more than 2^8; O_t and
-                // l are rescaled (P V of the previous key tile must be done)
-                auto maybe_raise = [&](float mx) {
-                    if (!__any_sync(0xffffffffu, mx > m_ref + 8.0f)) return false;
-                    const float m_new = fmaxf(m_ref, mx);
-                    const float alpha = exp2_fast(m_ref - m_new);
-                    m_ref = m_new;
-                    if (ensure_pv()) rescale(alpha);
-                    return true;
-                };
-                {
-                    float sv[64];
-                    load_half(0, sv);
-                    maybe_raise(half_max(sv));
-                    if (!ok) break;
-                    emit_half(0, sv);
-                    if (!ok) break;
-                }
-                {
-                    float sv[64];
-                    load_half(1, sv);
-                    const bool raised = maybe_raise(half_max(sv));
-                    if (!ok) break;
-                    if (raised) {
-                        // the first half's P is against the old max: redo it
-                        float sv0[64];
-                        load_half(0, sv0);
-                        emit_half(0, sv0);
-                        if (!ok) break;
-                    }
-                    // S_t fully read: the next key tile's S may overwrite it
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&s_free[t]);
-                    emit_half(1, sv);
-                    if (!ok) break;
-                }
-                tmem_wait_st();
-                l_run += (sum0.x + sum0.y) + (sum1.x + sum1.y);
-                tc_fence_before();  // P (and a rescaled O) written before P V may start
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&p_full[t]);
-            }
-            if (!ok) break;
-            g += (uint32_t)nkt;
-            // every P V of the item done: O_t / l, stored as bf16
-            if (!wait(&pv_done[t], (g - 1) & 1)) break;
+        const float scale = p.scale_log2;
+        const f32x2 sc2 = {scale, scale};
+        float m_ref = -INFINITY, l_run = 0.f;
+        // S_t of key tile g into registers; S_t is released at once, so the
+        // next key tile's S runs under this one's exponents
+        auto load_s = [&](uint32_t g, float (&sv)[128]) {
+            if (!wait(&s_full[t], g & 1)) return false;
             tc_fence_after();
-            float acc[DH];
+            uint32_t r[4][32];
 #pragma unroll
-            for (int d0 = 0; d0 < DH; d0 += 32) {
-                uint32_t r[32];
-                tmem_ld32(o_addr + d0, r);
-                tmem_wait_ld();
+            for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + 32 * c, r[c]);
+            tmem_wait_ld();
 #pragma unroll
-                for (int d = 0; d < 32; ++d) acc[d0 + d] = __uint_as_float(r[d]);
-            }
+            for (int c = 0; c < 128; ++c) sv[c] = __uint_as_float(r[c / 32][c % 32]);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&o_free[t]);
-            const int orow = it.q_row0 + 128 * t + row;
-            if (it.store[t] && orow < it.store_end) {
-                const float inv = 1.0f / l_run;
-                uint4 *dst = reinterpret_cast<uint4 *>(p.out + (size_t)orow * p.ldo + it.h * DH);
+            if (lane == 0) mbar_arrive(&s_free[t]);
+            return true;
+        };
+        // exponents of 64 scores against the reference -nm, their sum added to
+        // s0, s1, as bf16 pairs
+        auto exps = [&](const float (&sv)[128], int hb, float nm, f32x2 &s0, f32x2 &s1, uint32_t (&pw)[32]) {
+            const f32x2 nm2 = {nm, nm};
 #pragma unroll
-                for (int d = 0; d < DH; d += 8) {
-                    uint4 u;
-                    u.x = pack_bf16x2(acc[d] * inv, acc[d + 1] * inv);
-                    u.y = pack_bf16x2(acc[d + 2] * inv, acc[d + 3] * inv);
-                    u.z = pack_bf16x2(acc[d + 4] * inv, acc[d + 5] * inv);
-                    u.w = pack_bf16x2(acc[d + 6] * inv, acc[d + 7] * inv);
-                    dst[d / 8] = u;
+            for (int c = 0; c < 32; c += 2) {
+                const int k0 = 64 * hb + 2 * c;
+                const f32x2 x0 = ffma2({sv[k0], sv[k0 + 1]}, sc2, nm2);
+                const f32x2 x1 = ffma2({sv[k0 + 2], sv[k0 + 3]}, sc2, nm2);
+                const f32x2 e0 = {exp2_fast(x0.x), exp2_fast(x0.y)};
+                const f32x2 e1 = {exp2_fast(x1.x), exp2_fast(x1.y)};
+                s0 = fadd2(s0, e0);
+                s1 = fadd2(s1, e1);
+                pw[c] = pack_bf16x2(e0.x, e0.y);
+                pw[c + 1] = pack_bf16x2(e1.x, e1.y);
+            }
+        };
+        auto p_written = [&]() {
+            tmem_wait_st();
+            tc_fence_before();  // P (and a rescaled O) written before P V may start
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&p_full[t]);
+        };
+        // A key tile against the reference as it stands: no maximum, no check.
+        auto plain_tile = [&](uint32_t g) {
+            float sv[128];
+            if (!load_s(g, sv)) return false;
+            f32x2 s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
+            uint32_t pw0[32], pw1[32];
+            exps(sv, 0, -m_ref, s0, s1, pw0);
+            if (!wait(&pv_done[t], (g - 1) & 1)) return false;  // P_t read by P V of the previous key tile
+            tc_fence_after();
+            tmem_st32(p_addr, pw0);
+            exps(sv, 1, -m_ref, s0, s1, pw1);
+            tmem_st32(p_addr + 32, pw1);
+            l_run += (s0.x + s0.y) + (s1.x + s1.y);
+            p_written();
+            return true;
+        };
+        // A key tile with its maximum (of its `valid` first keys): the item's
+        // first and a ragged last one, and every one of a second pass.  The
+        // reference is raised (O_t and l rescaled) when it grew by more than 2^8.
+        auto max_tile = [&](uint32_t g, bool first, int valid) {
+            float sv[128];
+            if (!load_s(g, sv)) return false;
+            if (valid < 128) {
+#pragma unroll
+                for (int c = 0; c < 128; ++c)
+                    if (c >= valid) sv[c] = -INFINITY;
+            }
+            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int c = 0; c < 128; c += 8) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx4[e] = fmax3(mx4[e], sv[c + e], sv[c + 4 + e]);
+            }
+            const float mx = fmax3(mx4[0], mx4[1], fmaxf(mx4[2], mx4[3])) * scale;
+            if (g > 0 && !wait(&pv_done[t], (g - 1) & 1)) return false;  // P_t, O_t free
+            tc_fence_after();
+            if (__any_sync(0xffffffffu, mx > m_ref + 8.0f)) {
+                const float m_new = fmaxf(m_ref, mx);
+                const float alpha = exp2_fast(m_ref - m_new);
+                m_ref = m_new;
+                l_run *= alpha;
+                if (!first) {  // O_t holds this item's earlier tiles
+#pragma unroll 1
+                    for (int d0 = 0; d0 < DH; d0 += 16) {
+                        uint32_t r[16];
+                        tmem_ld16(o_addr + d0, r);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
+                        tmem_st16(o_addr + d0, r);
+                    }
                 }
             }
+            const float nm = m_ref == -INFINITY ? 0.f : -m_ref;
+            f32x2 s0 = {0.f, 0.f}, s1 = {0.f, 0.f};
+            uint32_t pw[2][32];
+            exps(sv, 0, nm, s0, s1, pw[0]);
+            exps(sv, 1, nm, s0, s1, pw[1]);
+            tmem_st32(p_addr, pw[0]);
+            tmem_st32(p_addr + 32, pw[1]);
+            l_run += (s0.x + s0.y) + (s1.x + s1.y);
+            p_written();
+            return true;
+        };
+        uint32_t g = 0;  // key tiles of this CTA's earlier items
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll 1
+            for (int w = blockIdx.x; w < total; w += gridDim.x) {
+                Item it;
+                const int nk = __shfl_sync(0xffffffffu, decode_item(p, w, n_tiles, it) ? it.nk : 0, 0);
+                if (nk == 0) continue;
+                m_ref = -INFINITY;
+                l_run = 0.f;
+                bool ok = true;
+#pragma unroll 1
+                for (int k0 = 0; k0 < nk && ok; k0 += 128, ++g) {
+                    if (k0 > 0 && nk - k0 >= 128 && pass == 0)
+                        ok = plain_tile(g);
+                    else
+                        ok = max_tile(g, k0 == 0, nk - k0);
+                }
+                if (!ok) break;
+                // every P V of the item done: O_t / l, stored as bf16
+                if (!wait(&pv_done[t], (g - 1) & 1)) break;
+                tc_fence_after();
+                float acc[DH];
+#pragma unroll
+                for (int d0 = 0; d0 < DH; d0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(o_addr + d0, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int d = 0; d < 32; ++d) acc[d0 + d] = __uint_as_float(r[d]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&o_free[t]);
+                const int orow = it.q_row0 + 128 * t + row;
+                if (it.store[t] && orow < it.store_end) {
+                    // The first pass takes the reference from the item's first
+                    // key tile.  P, l and O carry it exactly as long as no
+                    // exponent overflows (all three have 8 exponent bits), and
+                    // a later score 2^64 above it shows in l, a sum of
+                    // positive terms; anything not finite in O is looked at
+                    // again too.
+                    float zero = 0.f;
+#pragma unroll
+                    for (int d = 0; d < DH; ++d) zero = fmaf(acc[d], 0.f, zero);  // NaN if any is inf or NaN
+                    if (pass == 0 && !(l_run <= 0x1p64f && zero == 0.f)) *redo_flag = 1;
+                    const float inv = 1.0f / l_run;
+                    uint4 *dst = reinterpret_cast<uint4 *>(p.out + (size_t)orow * p.ldo + it.h * DH);
+#pragma unroll
+                    for (int d = 0; d < DH; d += 8) {
+                        uint4 u;
+                        u.x = pack_bf16x2(acc[d] * inv, acc[d + 1] * inv);
+                        u.y = pack_bf16x2(acc[d + 2] * inv, acc[d + 3] * inv);
+                        u.z = pack_bf16x2(acc[d + 4] * inv, acc[d + 5] * inv);
+                        u.w = pack_bf16x2(acc[d + 6] * inv, acc[d + 7] * inv);
+                        dst[d / 8] = u;
+                    }
+                }
+            }
+            if (!again()) break;
         }
     }
     __syncthreads();
     if (*abort_flag) {
-        if (warp == 1) {
+        if (warp == 1 || warp == 2) {
             mma_commit_elect(drain);  // the MMAs' issuing lane
             if (lane == 0) wait_bounded(drain, 0, 100000000ull);
         }

@@ -120,3 +120,42 @@ def test_attention_reference_max_raised_in_late_tiles(orc, nq, nk, H, dh):
     assert np.isfinite(got).all()
     assert rel_l2(got, ref) < 1e-2
     assert np.max(np.abs(got - ref)) < 2e-2
+
+
+@pytest.mark.parametrize("nq,nk,H,dh", [(1280, 900, 16, 64), (2600, 700, 8, 32)])
+@pytest.mark.parametrize("kind", ["scores", "values", "nan"])
+def test_attention_first_pass_reference_is_not_enough(orc, nq, nk, H, dh, kind):
+    # the pair kernel takes its reference from an item's first key tile and
+    # repeats a CTA's items with running maxima when that does not carry:
+    # scores 2^100 and 2^170 above the first tile's, values so large that
+    # 2^40 P overflows the fp32 accumulator, and a NaN query row (which must
+    # stay NaN and leave the other rows alone)
+    g = np.random.default_rng(nq + nk)
+    W = H * dh
+    u = np.where(g.random((H, dh)) < 0.5, -1.0, 1.0)
+    c = g.uniform(0.95, 1.0, nq)
+    q = np.einsum("r,hd->rhd", c, u).reshape(nq, W)
+    unit = 1.0 / (np.sqrt(dh) * np.log2(np.e))         # key strength worth one log2 unit of scaled score
+    up = {"scores": (100.0, 170.0), "values": (40.0, 40.0), "nan": (0.0, 0.0)}[kind]
+    a = np.zeros(nk)
+    a[256:384] = up[0] * unit
+    a[nk - 60:] = up[1] * unit
+    k = np.einsum("j,hd->jhd", a, u).reshape(nk, W) + 0.02 * g.standard_normal((nk, W))
+    v = g.standard_normal((nk, W)) * (1e30 if kind == "values" else 1.0)
+    if kind == "nan":
+        q[7, 3] = np.nan
+    qb, kb, vb = (synth.f32_to_bf16_bits(x.astype(np.float32)) for x in (q, k, v))
+    out = torch.zeros((nq, W), dtype=torch.bfloat16, device="cuda")
+    f3dc.attention(dev_bf16(qb), W, dev_bf16(kb), dev_bf16(vb), W, out, nq, nk, H, dh)
+    assert f3dc.gemm_status() == 0
+    rows = np.unique(np.concatenate([[0, 7, 127, 128, nq - 1], g.integers(0, nq, 24)]))
+    qf, kf, vf = (synth.bf16_bits_to_f32(x) for x in (qb, kb, vb))
+    got = out.float().cpu().numpy()[rows].astype(np.float64)
+    if kind == "nan":
+        assert np.isnan(got[rows == 7, :dh]).all() and np.isfinite(got[rows == 7, dh:]).all()
+        got, rows = got[rows != 7], rows[rows != 7]
+    ref = orc.attention(qf[rows], kf, vf, H).astype(np.float64)
+    scale = 1e30 if kind == "values" else 1.0
+    assert np.isfinite(got).all()
+    assert rel_l2(got / scale, ref / scale) < 1e-2
+    assert np.max(np.abs(got - ref)) / scale < 2e-2
