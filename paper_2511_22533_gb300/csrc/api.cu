@@ -1057,7 +1057,6 @@ f3dc_status f3dc_step(f3dc_handle *h, int32_t k, int32_t B, float *S_inout, void
         d.bits = h->dec_bits;
         d.compare = compare;
         d.dyn = dyn_voxels_dev;
-        d.num_sms = h->num_sms;
         return launch_decode_conv(d, s);
     };
     // (4D)^3 outputs of the last layer plus (2D)^3 x 8 and D^3 x 16 before it

@@ -503,7 +503,18 @@ F3DC_DEV f32x2 fadd2(f32x2 a, f32x2 b)
     uint64_t pa, pb, d;
     asm("mov.b64 %0, {%1, %2};" : "=l"(pa) : "f"(a.x), "f"(a.y));
     asm("mov.b64 %0, {%1, %2};" : "=l"(pb) : "f"(b.x), "f"(b.y));
-    asm("add.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pa), "l"(pb));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pa), "l"(pb));
+    f32x2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
+    return r;
+}
+
+F3DC_DEV f32x2 fmul2(f32x2 a, f32x2 b)
+{
+    uint64_t pa, pb, d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(pa) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(pb) : "f"(b.x), "f"(b.y));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pa), "l"(pb));
     f32x2 r;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(d));
     return r;

@@ -109,7 +109,6 @@ struct DecodeArgs {
     uint32_t *bits;                                // [B, 2 D^3]
     int compare;
     int64_t *dyn;                                  // [B] when compare
-    int num_sms;
 };
 size_t decode_scratch_floats(int B, int D);
 cudaError_t launch_decode_conv(const DecodeArgs &a, cudaStream_t s);

@@ -40,6 +40,12 @@ def test_anchor_step_dynamic_voxels_exact(orc, shape):
     h.close()
 
 
+@pytest.mark.parametrize("grid", [4, 12, 20])
+def test_anchor_step_dynamic_voxels_exact_on_odd_rows(orc, grid):
+    # grid rows that do not fill a warp (and 20^3: a last block that is not full)
+    test_anchor_step_dynamic_voxels_exact(orc, synth.ModelShape(grid, 8, 128, 1, 4, 4, 64, 128, 8, 64))
+
+
 def test_sampler_sigma_with_conv_decoder(orc):
     # Algorithm 1 measuring sigma with the convolutional decoder: both sides
     # decode nearly the same latents at the anchor step
