@@ -317,13 +317,14 @@ f3dc_status f3dc_forward(f3dc_handle *h, float t, int32_t B, const float *S,
 #define F3DC_EPI_RESID 2  /* out fp32 += gate * (acc + bias), gate nullable (1) */
 
 /* out[m, n] = epi(sum_k A[m, k] B[n, k]) -- the tcgen05 GEMM of the
- * transformer (nn.Linear convention: B is [N, K] row-major).  When the output
- * tiles (128 rows x 64/128/256 columns) would leave at least half of the SMs
- * idle and K >= 2048, the K range is split over several CTAs whose fp32
- * partials go to a split-K workspace that this call allocates once per device
- * and keeps for the life of the process; results do not depend on the split
- * (partials are summed in a fixed order), and calls on one device must not
- * overlap.  A bounded wait inside the kernel that runs out (F3DC_DEV_TIMEOUT;
+ * transformer (nn.Linear convention: B is [N, K] row-major).  N a multiple of
+ * 256 with K a multiple of 128 runs on CTA pairs (one launch, no workspace).
+ * Other shapes run on single CTAs: when their output tiles (128 rows x
+ * 64/128/256 columns) would leave at least half of the SMs idle and K >= 2048,
+ * the K range is split over several CTAs whose fp32 partials go to a split-K
+ * workspace that this call allocates once per device and keeps for the life of
+ * the process; results do not depend on the split (partials are summed in a
+ * fixed order), and calls on one device must not overlap.  A bounded wait inside the kernel that runs out (F3DC_DEV_TIMEOUT;
  * the output is then incomplete) is recorded in the device status word that
  * f3dc_gemm_status reads.
  *   A: device bf16 [M, K] row-major; B: device bf16 [N, K] row-major;
@@ -341,8 +342,8 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
  * latency-critical loops must not enter the driver's allocator; f3dc_gemm,
  * which allocates its split-K workspace on first use per device, serves none
  * of them.  This call makes f3dc_gemm's launch decisions (the CTA-pair kernel
- * for 256-wide tiles without a split, otherwise the single-CTA kernel with
- * the same split rule and summation order), so its output equals f3dc_gemm's
+ * where N and K allow, otherwise the single-CTA kernel with the same split
+ * rule and summation order), so its output equals f3dc_gemm's
  * bit for bit, with the same arguments and errors; but it takes the split-K
  * workspace from a fixed 20 MiB array (plus 4 KiB of counters) compiled into
  * libf3dc; every GPU that loads the library holds that array until the
@@ -387,7 +388,8 @@ f3dc_status f3dc_gemm_status(uint32_t *status_out);
  *     expects this many arrivals beyond the splits that exist (arrivals no CTA
  *     makes) and gives up after gemm_wait_ns nanoseconds (0: the default 1 s);
  *     the kernel then records F3DC_DEV_TIMEOUT (read with f3dc_gemm_status),
- *     leaves the waiting tiles unwritten and returns.  0 turns it off.
+ *     leaves the waiting tiles unwritten and returns.  While it is on, f3dc_gemm
+ *     takes the single-CTA kernel for every shape.  0 turns it off.
  *   attn_missing_kv: 1 makes f3dc_attention's first CTA skip the load of the
  *     last key tile of its first item, so the waits on that tile run out
  *     (after 1 s); the kernel records F3DC_DEV_TIMEOUT (read with

@@ -324,8 +324,18 @@ struct f3dc_handle {
     cudaStream_t exec_stream = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
 
-    CUtensorMap tm_h, tm_att, tm_u, tm_cond, tm_q_self, tm_q_cross;
-    std::vector<CUtensorMap> tm_qkv_w, tm_o_w, tm_cq_w, tm_co_w, tm_fc1_w, tm_fc2_w, tm_ckv_w, tm_kv_cross;
+    // a GEMM operand's tensor maps, for the kernel that its tile width takes
+    struct OperandA {
+        CUtensorMap one, pair;
+    };
+    struct OperandB {
+        CUtensorMap one;
+        GemmPairB pair;
+    };
+    OperandA tm_h, tm_att, tm_u, tm_cond;
+    CUtensorMap tm_q_self, tm_q_cross;
+    std::vector<OperandB> tm_qkv_w, tm_o_w, tm_cq_w, tm_co_w, tm_fc1_w, tm_fc2_w, tm_ckv_w;
+    std::vector<CUtensorMap> tm_kv_cross;
     int bn_qkv = 128, bn_w = 128, bn_fc1 = 128, bn_ckv = 128;
 
     const bf16 *wt(size_t off) const { return wblob + off; }
@@ -426,9 +436,6 @@ cudaError_t dalloc(T **p, size_t count)
     return cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T) + 256);
 }
 
-// B-operand box rows of a step weight: 256-wide GEMMs run on CTA pairs.
-uint32_t wide_b_box(int bn) { return bn == 256 ? kGemmPairBBox : gemm_b_box_rows(bn); }
-
 // Tile width of a step GEMM: the widest that divides N.  A 128 x 256 tile
 // needs 96 B of operands per clock of MMA against 128 B for 128 x 128, and
 // the operand stream from L2 into each SM is what bounds these GEMMs: at 4096
@@ -441,7 +448,7 @@ int pick_bn(int N)
     return 64;
 }
 
-cudaError_t run_gemm(f3dc_handle *h, const CUtensorMap &ta, const CUtensorMap &tb, int N, int K, int bn, int epi,
+cudaError_t run_gemm(f3dc_handle *h, const f3dc_handle::OperandA &ta, const f3dc_handle::OperandB &tb, int N, int K, int bn, int epi,
                      void *out, int ldo, const bf16 *bias, const float *gate, const bf16 *qn, const bf16 *kn,
                      cudaStream_t s)
 {
@@ -466,15 +473,14 @@ cudaError_t run_gemm(f3dc_handle *h, const CUtensorMap &ta, const CUtensorMap &t
     p.counters = h->gemm_cnt;
     p.ws_units = h->num_sms;
     p.err = h->dev_err;
-    // 256-wide tiles run on CTA pairs; those that would leave more than half
-    // of the SMs idle (few active rows) run 128 wide
-    if (bn == 256) {
-        p.narrow_below = h->num_sms / 2;
-        return launch_gemm_pair(&ta, &tb, p, epi, (h->max_tiles + 1) / 2 * (N / 128), s);
-    }
+    // 256-wide tiles run on CTA pairs.  At most one cluster per 128 columns: a
+    // model whose launches are all small (8^3 grid, width 128) is bound by their
+    // latency, and its sample takes 1017 us with 16-CTA launches of fc1, 1036
+    // with 32 (64-column units)
+    if (bn == 256) return launch_gemm_pair(&ta.pair, &tb.pair, p, epi, (h->max_tiles + 1) / 2 * (N / 128), s);
     const int tiles = h->max_tiles * (N / bn);
     const int grid = tiles < h->num_sms ? tiles : h->num_sms;
-    return launch_gemm(&ta, &tb, p, epi, bn, grid, s);
+    return launch_gemm(&ta.one, &tb.one, p, epi, bn, grid, s);
 }
 
 cudaError_t run_attention(f3dc_handle *h, int mode, const CUtensorMap &tq, const CUtensorMap &tkv, int q_col0,
@@ -654,8 +660,15 @@ bool build_maps(f3dc_handle *h)
 {
     const int W = h->W, Wm = h->Wm, dh = h->dh;
     const uint64_t R = (uint64_t)h->max_rows;
-    bool ok = make_tmap_bf16(&h->tm_h, h->h, R, W, W, 128, 64) && make_tmap_bf16(&h->tm_att, h->att, R, W, W, 128, 64) &&
-              make_tmap_bf16(&h->tm_u, h->u, R, Wm, Wm, 128, 64) &&
+    auto act = [&](f3dc_handle::OperandA &m, const bf16 *base, int K) {
+        return make_tmap_bf16(&m.one, base, R, K, K, 128, 64) && make_tmap_pair(&m.pair, base, R, K, 128);
+    };
+    // a weight [N, K] in the form of the kernel that runs it (bn 256: CTA pairs)
+    auto weight = [&](f3dc_handle::OperandB &m, size_t off, int N, int K, int bn) {
+        return bn == 256 && K % 128 == 0 ? make_tmap_pair_b(&m.pair, h->wt(off), N, K)
+                                         : make_tmap_bf16(&m.one, h->wt(off), N, K, K, gemm_b_box_rows(bn), 64);
+    };
+    bool ok = act(h->tm_h, h->h, W) && act(h->tm_att, h->att, W) && act(h->tm_u, h->u, Wm) &&
               make_tmap_bf16(&h->tm_q_self, h->qkv, R, 3 * W, 3 * W, 128, dh) &&
               make_tmap_bf16(&h->tm_q_cross, h->qc, R, W, W, 128, dh);
     if (!ok) return false;
@@ -670,14 +683,10 @@ bool build_maps(f3dc_handle *h)
     h->tm_kv_cross.resize(L);
     for (int l = 0; l < L; ++l) {
         const BlockOffsets &b = h->lay.blk[l];
-        ok = ok && make_tmap_bf16(&h->tm_qkv_w[l], h->wt(b.qkv_w), 3 * W, W, W, wide_b_box(h->bn_qkv), 64);
-        ok = ok && make_tmap_bf16(&h->tm_o_w[l], h->wt(b.o_w), W, W, W, wide_b_box(h->bn_w), 64);
-        ok = ok && make_tmap_bf16(&h->tm_cq_w[l], h->wt(b.cq_w), W, W, W, wide_b_box(h->bn_w), 64);
-        ok = ok && make_tmap_bf16(&h->tm_co_w[l], h->wt(b.co_w), W, W, W, wide_b_box(h->bn_w), 64);
-        ok = ok && make_tmap_bf16(&h->tm_fc1_w[l], h->wt(b.fc1_w), Wm, W, W, wide_b_box(h->bn_fc1), 64);
-        ok = ok && make_tmap_bf16(&h->tm_fc2_w[l], h->wt(b.fc2_w), W, Wm, Wm, wide_b_box(h->bn_w), 64);
-        ok = ok && make_tmap_bf16(&h->tm_ckv_w[l], h->wt(b.ckv_w), 2 * W, h->Dc, h->Dc,
-                                  h->Dc % 128 == 0 ? wide_b_box(h->bn_ckv) : gemm_b_box_rows(h->bn_ckv), 64);
+        ok = ok && weight(h->tm_qkv_w[l], b.qkv_w, 3 * W, W, h->bn_qkv) && weight(h->tm_o_w[l], b.o_w, W, W, h->bn_w) &&
+             weight(h->tm_cq_w[l], b.cq_w, W, W, h->bn_w) && weight(h->tm_co_w[l], b.co_w, W, W, h->bn_w) &&
+             weight(h->tm_fc1_w[l], b.fc1_w, Wm, W, h->bn_fc1) && weight(h->tm_fc2_w[l], b.fc2_w, W, Wm, h->bn_w) &&
+             weight(h->tm_ckv_w[l], b.ckv_w, 2 * W, h->Dc, h->bn_ckv);
         ok = ok && make_tmap_bf16(&h->tm_kv_cross[l], h->ckv + (size_t)l * h->ckv_rows * 2 * W, h->ckv_rows, 2 * W,
                                   2 * W, 128, dh);
     }
@@ -995,7 +1004,9 @@ f3dc_status f3dc_set_cond(f3dc_handle *h, const void *cond, int32_t B, void *str
     cudaStream_t s = (cudaStream_t)stream;
     h->last_stream = s;
     const int rows = B * h->Nc;
-    if (!make_tmap_bf16(&h->tm_cond, cond, rows, h->Dc, h->Dc, 128, 64))
+    const bool pair = h->bn_ckv == 256 && h->Dc % 128 == 0;
+    if (!(pair ? make_tmap_pair(&h->tm_cond.pair, cond, rows, h->Dc, 128)
+               : make_tmap_bf16(&h->tm_cond.one, cond, rows, h->Dc, h->Dc, 128, 64)))
         return fail(h, F3DC_ERR_CUDA, "cuTensorMapEncodeTiled failed for cond");
     for (int l = 0; l < h->L; ++l) {
         GemmParams p;
@@ -1009,13 +1020,12 @@ f3dc_status f3dc_set_cond(f3dc_handle *h, const void *cond, int32_t B, void *str
         p.bias = h->wt(h->lay.blk[l].ckv_b);
         p.err = h->dev_err;
         const int tiles = p.m_tiles * (p.N / h->bn_ckv);
-        if (h->bn_ckv == 256 && h->Dc % 128 == 0) {
-            p.narrow_below = h->num_sms / 2;
+        if (pair) {
             LAUNCH(KF_GEMM_COND, wfix(2.0 * rows * p.N * (double)p.K, true),
-                   launch_gemm_pair(&h->tm_cond, &h->tm_ckv_w[l], p, kEpiBias, (p.m_tiles + 1) / 2 * (p.N / 128), s));
+                   launch_gemm_pair(&h->tm_cond.pair, &h->tm_ckv_w[l].pair, p, kEpiBias, (p.m_tiles + 1) / 2 * (p.N / 128), s));
         } else {
             LAUNCH(KF_GEMM_COND, wfix(2.0 * rows * p.N * (double)p.K, true),
-                   launch_gemm(&h->tm_cond, &h->tm_ckv_w[l], p, kEpiBias, h->bn_ckv,
+                   launch_gemm(&h->tm_cond.one, &h->tm_ckv_w[l].one, p, kEpiBias, h->bn_ckv,
                                tiles < h->num_sms ? tiles : h->num_sms, s));
         }
     }
@@ -1422,12 +1432,12 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int m_tiles = (M + kTileRows - 1) / kTileRows;
-    // 256-wide tiles without split K run on CTA pairs
-    const bool pair = bn == 256 && K % 128 == 0 && gemm_split_count(m_tiles * (N / bn), gemm_grid(m_tiles * (N / bn), sms), K / 64,
-                                                    sms, true) == 1;
+    // the injected missing arrival is the split-K kernel's
+    const bool pair = gemm_on_pairs(N, K) && fault_injection().gemm_missing_arrivals == 0;
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, A, M, K, K, 128, 64) ||
-        !make_tmap_bf16(&tb, B, N, K, K, pair ? kGemmPairBBox : gemm_b_box_rows(bn), 64))
+    GemmPairB tbp;
+    if (!(pair ? make_tmap_pair(&ta, A, M, K, 128) && make_tmap_pair_b(&tbp, B, N, K)
+               : make_tmap_bf16(&ta, A, M, K, K, 128, 64) && make_tmap_bf16(&tb, B, N, K, K, gemm_b_box_rows(bn), 64)))
         return fail(nullptr, F3DC_ERR_INVALID_ARG, "cuTensorMapEncodeTiled rejected A or B (alignment?)");
     GemmParams p;
     memset(&p, 0, sizeof(p));
@@ -1445,9 +1455,14 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     const int tiles = p.m_tiles * (N / bn);
     const int epi = epilogue == F3DC_EPI_BIAS ? kEpiBias : (epilogue == F3DC_EPI_GELU ? kEpiGelu : kEpiResid);
     cudaStream_t s = (cudaStream_t)stream;
+    const bool split = gemm_split_count(tiles, gemm_grid(tiles, sms), K / 64, sms, true) > 1;
     if (pair) {
-        p.narrow_below = sms / 2;
-        CK(launch_gemm_pair(&ta, &tb, p, epi, (m_tiles + 1) / 2 * (N / 128), s));
+        p.pieces = split;
+        CK(launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s));
+        return F3DC_OK;
+    }
+    if (!split) {
+        CK(launch_gemm(&ta, &tb, p, epi, bn, tiles < sms ? tiles : sms, s));
         return F3DC_OK;
     }
     // split-K workspace: allocated once per device on first use and kept for

@@ -145,6 +145,13 @@ F3DC_DEV void tma_prefetch_l2_2d(const CUtensorMap *map, int x, int y)
                  : "memory");
 }
 
+F3DC_DEV void tma_prefetch_l2_3d(const CUtensorMap *map, int x, int y, int z)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"((uint64_t)map), "r"(x),
+                 "r"(y), "r"(z)
+                 : "memory");
+}
+
 // Tiled TMA store of a shared-memory box to global memory (bulk-group
 // completion), and the same as an element-wise fp32 add into global memory.
 // Coordinates: x = innermost (column), y = row; the box is clipped at the
@@ -242,14 +249,14 @@ F3DC_DEV void mbar_arrive_cluster(uint32_t cluster_addr)
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
-// TMA load into this CTA's shared memory whose completion is counted on an
-// mbarrier of either CTA of the pair (shared::cluster address)
-F3DC_DEV void tma_load_2d_pair(void *smem_dst, const CUtensorMap *map, int x, int y, uint32_t bar_cluster)
+// TMA load of a 3-D box into this CTA's shared memory whose completion is
+// counted on an mbarrier of either CTA of the pair (shared::cluster address)
+F3DC_DEV void tma_load_3d_pair(void *smem_dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar_cluster)
 {
     asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(smem_dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar_cluster)
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(smem_dst)),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
         : "memory");
 }
 
@@ -334,6 +341,26 @@ F3DC_DEV void mma_bf16_pair_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_d
         "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
         " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The eight pair MMAs of 128 K (two 64-K regions of each operand, a_half and
+// b_half apart in descriptor units; 16 K further is 2 units) under one election.
+F3DC_DEV void mma_bf16_pair_128k(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint64_t a_half, uint64_t b_half,
+                                 uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n .reg .pred p, e, t;\n .reg .b64 a, b;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %6, 0;\n setp.eq.b32 t, 0, 0;\n"
+        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %5, p;\n"
+        " add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, a, 2;\n add.s64 b, b, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, a, 2;\n add.s64 b, b, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, %1, %3;\n add.s64 b, %2, %4;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, a, 2;\n add.s64 b, b, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, a, 2;\n add.s64 b, b, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        " add.s64 a, a, 2;\n add.s64 b, b, 2;\n @e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, t;\n"
+        "}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "l"(a_half), "l"(b_half), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 

@@ -108,6 +108,29 @@ struct TmemSrc {
     }
 };
 
+// Adds accumulators 1 .. n - 1 (bn TMEM columns apart) to accumulator 0 in
+// order, in the 32-column chunks k0, k0 + kstep, ... of this warp's lanes.
+F3DC_DEV void sum_accumulators(uint32_t tbase, int bn, int n, int k0, int kstep)
+{
+#pragma unroll 1
+    for (int c0 = 32 * k0; c0 < bn; c0 += 32 * kstep) {
+        float v[32];
+        TmemSrc{tbase}(c0, v);
+#pragma unroll 1
+        for (int a = 1; a < n; ++a) {
+            float w[32];
+            TmemSrc{tbase + (uint32_t)(a * bn)}(c0, w);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += w[j];
+        }
+        uint32_t r[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
+        tmem_st32(tbase + c0, r);
+    }
+    tmem_wait_st();
+}
+
 template <int BN>
 struct WsSrc {
     const float *ws;  // partials of split s of this tile: unit (s * tiles + tile), chunk-major
@@ -384,12 +407,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     griddep_wait();
     Units U;
     U.m_tiles = p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles;
-    // narrow mode: a 256-wide kernel whose tile count would leave too many SMs
-    // idle (the row count is only known here) runs 128-wide tiles instead,
-    // with the same stages (half of each B stage used) and TMEM buffers
-    const bool narrow = BN == 256 && p.ws == nullptr && U.m_tiles * (p.N / BN) < p.narrow_below;
-    const int bn = narrow ? BN / 2 : BN;
-    U.tiles = U.m_tiles * (p.N / bn);
+    U.tiles = U.m_tiles * (p.N / BN);
     U.kb_n = p.K / kBK;
     U.splits = gemm_split_count(U.tiles, (int)gridDim.x, U.kb_n, p.ws_units, p.ws != nullptr);
     U.kb_per = (U.kb_n + U.splits - 1) / U.splits;
@@ -405,17 +423,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             bool ok = true;
             for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
                 int m0, n0, kb0, kb1;
-                U.decode(t, m0, n0, kb0, kb1, bn);
+                U.decode(t, m0, n0, kb0, kb1, BN);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&full[s], kAStage + bn * kBK * 2);
+                    mbar_arrive_expect_tx(&full[s], kAStage + BN * kBK * 2);
                     tma_load_2d(sa + s * kAStage, &tma, kb * kBK, m0, &full[s]);
                     // B in boxes of kBBox rows, stacked in the stage (the
                     // 8-row swizzle atoms continue across boxes)
-                    for (int hb = 0; hb < bn; hb += kBBox)
+                    for (int hb = 0; hb < BN; hb += kBBox)
                         tma_load_2d(sb + s * Cfg::kBStage + hb * (kBK * 2), &tmb, kb * kBK, n0 + hb, &full[s]);
                     if (++s == S) {
                         s = 0;
@@ -432,9 +450,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         // The whole warp runs the loop (barrier outcomes as warp votes) and
         // elect.sync issues.
         {
-            constexpr uint32_t idesc_w = make_idesc_bf16(128, BN, 0, 0);
-            constexpr uint32_t idesc_n = make_idesc_bf16(128, BN / 2 < 16 ? 16 : BN / 2, 0, 0);
-            const uint32_t idesc = narrow ? idesc_n : idesc_w;
+            constexpr uint32_t idesc = make_idesc_bf16(128, BN, 0, 0);
             // stage-0 descriptors; stage s adds s * stage bytes / 16, a K
             // step of 16 elements inside the 128B swizzle atom adds 2
             const uint64_t a_desc0 = make_sdesc(smem_u32(sa), 16, 1024, kSwizzle128);
@@ -451,7 +467,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     break;
                 const uint32_t d = tmem + buf * BN;
                 int m0, n0, kb0, kb1;
-                U.decode(t, m0, n0, kb0, kb1, bn);
+                U.decode(t, m0, n0, kb0, kb1, BN);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ready && !warp_all(mbar_wait(&full[s], ph, abort_flag, p.err))) {
                         ok = false;
@@ -494,10 +510,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             if (!all) break;
             tc_fence_after();
             int m0, n0, kb0, kb1;
-            U.decode(t, m0, n0, kb0, kb1, bn);
+            U.decode(t, m0, n0, kb0, kb1, BN);
             const TmemSrc tsrc{tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN)};
             if (U.splits == 1) {
-                epilogue_tile<EPI>(p, tsrc, o, m0, n0, bn);
+                epilogue_tile<EPI>(p, tsrc, o, m0, n0, BN);
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acce[buf]);
@@ -588,7 +604,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
 // ------------------------------------------------------------ CTA pair
 // cta_group::2 GEMM for 256-wide tiles.  A cluster of two CTAs computes a
-// 256 x 256 tile (256 x 128 in narrow mode): each CTA loads its 128 rows of A
+// 256 x 256 tile (a launch's last wave 256 x 128 or 256 x 64): each CTA loads its 128 rows of A
 // and its half of the tile's B rows into its own shared memory (128 K per stage), the even CTA
 // issues the 256-row MMAs for both, and each CTA's TMEM receives its own 128
 // rows of the accumulator, which its epilogue warps write out.  Per SM that
@@ -616,9 +632,52 @@ constexpr int kPairOutBufs = 2;
 constexpr size_t kPairSmem = 1024 + (size_t)kPairStages * (kPairAStage + kPairBStage) +
                              2 * (size_t)kPairOutBufs * kOutChunkBytes + 256;
 
+// Work units of a launch whose row count is only known on the device: full
+// waves of 256-wide tiles, and the tiles left for the last wave cut into 2 or 4
+// units of 128 or 64 columns when that many clusters are free for them (a
+// launch of less than half a wave is all last wave).  A narrower unit costs
+// more operand bytes per product (its 256 rows of A are read for fewer
+// columns), so it only pays on clusters that would idle: 1229 x 4096 x 1024
+// (80 tiles on 76 clusters) 16.2 -> 12.7 us, 4096 x 4096 x 1024 27.7 -> 24.0.
+// Units run column-fastest: the weights (8 MB at most here) stay in L2 and each
+// row block of A is read from memory once, also when A is larger than L2
+// (25000 x 1024 x 4096: 177 us row-fastest, 130).
+struct PairUnits {
+    int n_tiles, full, sub, total;  // column tiles; full-width units; pieces of each other tile; units
+    float inv_n;
+    F3DC_DEV PairUnits(int pm_tiles, int N, int clusters, int rows)
+    {
+        n_tiles = N / 256;
+        inv_n = 1.0f / (float)n_tiles;
+        const int tiles = pm_tiles * n_tiles;
+        full = tiles / clusters * clusters;
+        const int rest = tiles - full;
+        // a handful of rows is read by every cluster from the same few L2 lines:
+        // more clusters wait longer (1 x 4096 x 1024: 10.5 us on 64 clusters, 8.9 on 32)
+        sub = 4 * rest <= clusters && rows >= 64 ? 4 : (2 * rest <= clusters ? 2 : 1);
+        total = full + rest * sub;
+    }
+    // unit u: row pair m, first column n0, width bn
+    F3DC_DEV void decode(int u, int &m, int &n0, int &bn) const
+    {
+        int tile = u, piece = 0;
+        bn = 256;
+        if (u >= full) {
+            const int v = u - full, log_sub = sub >> 1;  // sub is 1, 2 or 4
+            tile = full + (v >> log_sub);
+            piece = v & (sub - 1);
+            bn = 256 >> log_sub;
+        }
+        // tile / n_tiles: the quotient's distance to an integer is at least
+        // 0.5 / n_tiles, the rounding error below tile / n_tiles * 2^-22
+        m = (int)(((float)tile + 0.5f) * inv_n);
+        n0 = (tile - m * n_tiles) * 256 + piece * bn;
+    }
+};
+
 template <int EPI>
 __global__ void __launch_bounds__(kPairThreads, 1)
-    k_gemm_pair(const __grid_constant__ CUtensorMap tma, const __grid_constant__ CUtensorMap tmb,
+    k_gemm_pair(const __grid_constant__ CUtensorMap tma, const __grid_constant__ GemmPairB tmb,
                 const __grid_constant__ CUtensorMap tmo, const GemmParams p)
 {
     constexpr int S = kPairStages;
@@ -632,11 +691,20 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_rank();
+    // warp-uniform values go through a shuffle where the compiler cannot see
+    // that they are
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t rank = __shfl_sync(0xffffffffu, cluster_rank(), 0);
     griddep_launch();
 
+    if (threadIdx.x == 64) {
+        // the descriptors are parameters: fetched while the barriers are set up
+        tma_prefetch(&tma);
+        for (int i = 0; i < 3; ++i) tma_prefetch(&tmb.rows[i]);
+        tma_prefetch(&tmo);
+    }
     if (threadIdx.x == 0) {
+#pragma unroll 1
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
@@ -653,40 +721,48 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         tmem_alloc_pair(tmem_holder, kPairTmemCols);
         tmem_relinquish_pair();
     }
-    if (warp == 0 && lane == 0) {
-        // the weights are constant: pull this CTA's share of B into L2 while
-        // the previous kernel finishes, so the first stages' loads hit L2
-        const int kbx = p.K / 64, boxes = (p.N / (int)kGemmPairBBox) * kbx;
-        for (int i = blockIdx.x; i < boxes; i += gridDim.x)
-            tma_prefetch_l2_2d(&tmb, (i % kbx) * 64, (i / kbx) * (int)kGemmPairBBox);
-    }
     tc_fence_before();
-    __syncthreads();
     cluster_sync();  // both CTAs' barriers are initialised before any remote signal
     tc_fence_after();
-    const uint32_t tmem = *tmem_holder;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
+    if (warp == 3 && lane == 0) {
+        // the weights are constant: pull this CTA's share of B into L2 while
+        // the previous kernel finishes, so the first stages' loads hit L2
+        const int kbx = p.K / kPairBK, boxes = (p.N / 128) * kbx;
+#pragma unroll 1
+        for (int i = blockIdx.x; i < boxes; i += gridDim.x)
+            tma_prefetch_l2_3d(&tmb.rows[0], 0, (i / kbx) * 128, (i % kbx) * 2);
+    }
     griddep_wait();
-    const int m_tiles = p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles;
-    const bool narrow = m_tiles * (p.N / 256) < p.narrow_below;
-    const int bn = narrow ? 128 : 256;  // tile width; this CTA holds bn / 2 B rows
-    const int pm_tiles = (m_tiles + 1) / 2;
-    const int tiles = pm_tiles * (p.N / bn);
+    const int m_tiles = __shfl_sync(0xffffffffu, p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles, 0);
     const int kb_n = p.K / kPairBK;
     const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+    const PairUnits U((m_tiles + 1) / 2, p.N, ncl, p.M);
+    // The tensor core truncates as it accumulates, so the error of a sum grows
+    // with its length (4096: 3.2e-6 relative, 1024: 7e-7).  A long K is summed
+    // in pieces where the second TMEM buffer is not needed for a next unit:
+    // as many accumulators as fit in TMEM, added in fp32 by the epilogue.  Only
+    // for fp32 results: a bf16 one rounds at 2^-9.
+    const int chunks = EPI == kEpiResid && p.pieces && U.total <= ncl ? (int)kPairTmemCols / (U.full ? 256 : 256 / U.sub) : 1;
+    const uint32_t chunk_kb = (uint32_t)((kb_n + chunks - 1) / chunks);
+    const int n_acc = (kb_n + (int)chunk_kb - 1) / (int)chunk_kb;
     const uint32_t full_c = mapa_shared(smem_u32(full), 0);  // the even CTA's full[0]
     const uint32_t acce_c = mapa_shared(smem_u32(acce), 0);
 
     if (warp == 0) {
         if (lane == 0) {
-            tma_prefetch(&tma);
-            tma_prefetch(&tmb);
-            const uint32_t stage_bytes = 2u * (kPairAStage + (uint32_t)(bn / 2) * kPairBK * 2);  // both CTAs
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
-            for (int t = cl; t < tiles && ok; t += ncl) {
-                const int arow = (t % pm_tiles) * 256 + (int)rank * 128;
-                const int brow = (t / pm_tiles) * bn + (int)rank * (bn / 2);
+#pragma unroll 1
+            for (int t = cl; t < U.total && ok; t += ncl) {
+                int m, n0, bn;  // this CTA holds bn / 2 of the unit's B rows
+                U.decode(t, m, n0, bn);
+                const int arow = m * 256 + (int)rank * 128;
+                const int brow = n0 + (int)rank * (bn / 2);
+                const CUtensorMap *mb = &tmb.rows[bn == 256 ? 0 : (bn == 128 ? 1 : 2)];
+                const uint32_t stage_bytes = 2u * (kPairAStage + (uint32_t)(bn / 2) * kPairBK * 2);  // both CTAs
+#pragma unroll 1
                 for (int kb = 0; kb < kb_n; ++kb) {
                     if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.err)) {
                         ok = false;
@@ -694,13 +770,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     }
                     if (rank == 0) mbar_arrive_expect_tx(&full[s], stage_bytes);
                     const uint32_t fb = full_c + 8u * (uint32_t)s;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int x = kb * kPairBK + h * 64;
-                        tma_load_2d_pair(sa + s * kPairAStage + h * kPairHalf, &tma, x, arow, fb);
-                        for (int hb = 0; hb < bn / 2; hb += (int)kGemmPairBBox)
-                            tma_load_2d_pair(sb + s * kPairBStage + h * kPairHalf + hb * 128, &tmb, x, brow + hb, fb);
-                    }
+                    tma_load_3d_pair(sa + s * kPairAStage, &tma, 0, arow, 2 * kb, fb);
+                    tma_load_3d_pair(sb + s * kPairBStage, mb, 0, brow, 2 * kb, fb);
                     if (++s == S) {
                         s = 0;
                         ph ^= 1;
@@ -712,22 +783,25 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         // the even CTA's warp issues for the pair: the whole warp runs the
         // loop (barrier outcomes as warp votes) and elect.sync issues
         if (rank == 0) {
-            constexpr uint32_t idesc_w = make_idesc_bf16(256, 256, 0, 0);
-            constexpr uint32_t idesc_n = make_idesc_bf16(256, 128, 0, 0);
-            const uint32_t idesc = narrow ? idesc_n : idesc_w;
             const uint64_t a_desc0 = make_sdesc(smem_u32(sa), 16, 1024, kSwizzle128);
             const uint64_t b_desc0 = make_sdesc(smem_u32(sb), 16, 1024, kSwizzle128);
             int s = 0, it = 0;
             uint32_t ph = 0;
             bool ok = true;
             bool ready = warp_all(mbar_test(&full[0], 0));
-            for (int t = cl; t < tiles && ok; t += ncl, ++it) {
+#pragma unroll 1
+            for (int t = cl; t < U.total && ok; t += ncl, ++it) {
+                const int bn = t < U.full ? 256 : 256 / U.sub;
+                const uint32_t idesc = make_idesc_bf16(256, bn, 0, 0);
+                const uint64_t b_half = (uint64_t)(bn / 2 * 128) >> 4;  // from a stage's first 64 K of B to the second
                 const int buf = it & 1;
                 const uint32_t aph = (it >> 1) & 1;
                 if (!warp_all(mbar_test(&acce[buf], aph ^ 1)) &&
                     !warp_all(mbar_wait(&acce[buf], aph ^ 1, abort_flag, p.err)))
                     break;
-                const uint32_t d = tmem + buf * 256;
+                uint32_t d = tmem + buf * 256, left = chunk_kb;
+                bool first = true;
+#pragma unroll 1
                 for (int kb = 0; kb < kb_n; ++kb) {
                     if (!ready && !warp_all(mbar_wait(&full[s], ph, abort_flag, p.err))) {
                         ok = false;
@@ -739,12 +813,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     ready = warp_all(mbar_test(&full[s_next], ph_next));
                     const uint64_t ad = a_desc0 + (uint64_t)s * (kPairAStage >> 4);
                     const uint64_t bd = b_desc0 + (uint64_t)s * (kPairBStage >> 4);
-#pragma unroll
-                    for (int k = 0; k < kPairBK / 16; ++k) {
-                        const uint64_t off = (uint64_t)(k >> 2) * (kPairHalf >> 4) + 2 * (k & 3);
-                        mma_bf16_pair_elect(d, ad + off, bd + off, idesc, (kb != 0) || (k != 0));
-                    }
+                    mma_bf16_pair_128k(d, ad, bd, kPairHalf >> 4, b_half, idesc, !first);
                     mma_commit_pair_mc_elect(&empty[s], 3);
+                    first = --left == 0;
+                    if (first) {  // the next accumulator
+                        d += bn;
+                        left = chunk_kb;
+                    }
                     s = s_next;
                     ph = ph_next;
                 }
@@ -757,10 +832,12 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         const int grp = (warp - 2) >> 2;
         OutStage o{so + grp * kPairOutBufs * kOutChunkBytes, &tmo, row, 0, kPairOutBufs, 3 + grp, 64 + 128 * grp};
         int it = 0;
-        for (int t = cl; t < tiles; t += ncl, ++it) {
+#pragma unroll 1
+        for (int t = cl; t < U.total; t += ncl, ++it) {
             const int buf = it & 1;
             const uint32_t aph = (it >> 1) & 1;
-            const int n0 = (t / pm_tiles) * bn;
+            int m, n0, bn;
+            U.decode(t, m, n0, bn);
             ColOps first;
             if constexpr (EPI != kEpiQKNorm) load_colops<EPI>(p, n0 + 32 * grp, first);
             const uint32_t got = mbar_wait(&accf[buf], aph, abort_flag, p.err) ? 1u : 0u;
@@ -772,12 +849,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                          : "memory");
             if (!all) break;
             tc_fence_after();
-            const int m0 = (t % pm_tiles) * 256 + (int)rank * 128;
+            const int m0 = m * 256 + (int)rank * 128;
             // the odd CTA's rows of the last pair lie beyond the plan when
             // the tile count is odd: computed, not stored
             if (m0 < m_tiles * 128) {
-                const TmemSrc tsrc{tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256)};
-                epilogue_tile<EPI>(p, tsrc, o, m0, n0, bn, grp, 2, &first);
+                const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256);
+                if (EPI == kEpiResid && n_acc > 1) sum_accumulators(acc, bn, n_acc, grp, 2);
+                epilogue_tile<EPI>(p, TmemSrc{acc}, o, m0, n0, bn, grp, 2, &first);
             }
             tc_fence_before();
             __syncwarp();
@@ -804,8 +882,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
 }
 
 template <int EPI>
-cudaError_t launch_pair_one(const CUtensorMap *ta, const CUtensorMap *tb, const CUtensorMap *to, const GemmParams &p,
-                            int max_pair_tiles, cudaStream_t s)
+cudaError_t launch_pair_one(const CUtensorMap *ta, const GemmPairB *tb, const CUtensorMap *to, const GemmParams &p,
+                            int max_units, cudaStream_t s)
 {
     // per device: the shared-memory attribute and the resident-cluster count
     // are taken on each device's first launch (0 = not yet known)
@@ -835,7 +913,7 @@ cudaError_t launch_pair_one(const CUtensorMap *ta, const CUtensorMap *tb, const 
         max_clusters = n;
         max_clusters_of[dev & 63].store(n, std::memory_order_release);
     }
-    const int clusters = max_pair_tiles < max_clusters ? (max_pair_tiles > 0 ? max_pair_tiles : 1) : max_clusters;
+    const int clusters = max_units < max_clusters ? (max_units > 0 ? max_units : 1) : max_clusters;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * clusters);
     cfg.blockDim = dim3(kPairThreads);
@@ -956,20 +1034,39 @@ cudaError_t launch_gemm(const CUtensorMap *ta, const CUtensorMap *tb, const Gemm
     }
 }
 
-cudaError_t launch_gemm_pair(const CUtensorMap *ta, const CUtensorMap *tb, const GemmParams &p, int epi,
-                             int max_pair_tiles, cudaStream_t s)
+cudaError_t launch_gemm_pair(const CUtensorMap *ta, const GemmPairB *tb, const GemmParams &p, int epi, int max_units,
+                             cudaStream_t s)
 {
     if (p.K % kPairBK != 0 || p.N % 256 != 0 || p.ws) return cudaErrorInvalidValue;
     CUtensorMap to;
     if (!make_tmap_out(&to, p.out, (uint64_t)p.M, (uint64_t)p.N, (uint64_t)p.ldo, epi == kEpiResid))
         return cudaErrorInvalidValue;
     switch (epi) {
-    case kEpiBias: return launch_pair_one<kEpiBias>(ta, tb, &to, p, max_pair_tiles, s);
-    case kEpiGelu: return launch_pair_one<kEpiGelu>(ta, tb, &to, p, max_pair_tiles, s);
-    case kEpiResid: return launch_pair_one<kEpiResid>(ta, tb, &to, p, max_pair_tiles, s);
-    case kEpiQKNorm: return launch_pair_one<kEpiQKNorm>(ta, tb, &to, p, max_pair_tiles, s);
+    case kEpiBias: return launch_pair_one<kEpiBias>(ta, tb, &to, p, max_units, s);
+    case kEpiGelu: return launch_pair_one<kEpiGelu>(ta, tb, &to, p, max_units, s);
+    case kEpiResid: return launch_pair_one<kEpiResid>(ta, tb, &to, p, max_units, s);
+    case kEpiQKNorm: return launch_pair_one<kEpiQKNorm>(ta, tb, &to, p, max_units, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+bool make_tmap_pair(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, uint32_t box_rows)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 encode = tmap_encoder();
+    if (!encode || ((uintptr_t)base & 15) != 0 || K % 128 != 0) return false;
+    cuuint64_t dims[3] = {64, rows, K / 64};
+    cuuint64_t strides[2] = {K * 2, 128};
+    cuuint32_t box[3] = {64, box_rows, 2};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_tmap_pair_b(GemmPairB *maps, const void *base, uint64_t rows, uint64_t K)
+{
+    return make_tmap_pair(&maps->rows[0], base, rows, K, 128) && make_tmap_pair(&maps->rows[1], base, rows, K, 64) &&
+           make_tmap_pair(&maps->rows[2], base, rows, K, 32);
 }
 
 bool make_tmap_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,

@@ -153,9 +153,10 @@ struct GemmParams {
     float *ws;
     int32_t *counters;
     int ws_units;             // partial tiles the workspace holds
-    // bn = 256 without a workspace: when the device-side tile count of
-    // 256-wide tiles is below this, the kernel runs 128-wide tiles (0: never)
-    int narrow_below;
+    // CTA pairs, RESID: sum a long K in pieces (several accumulators, added in
+    // fp32) where TMEM has room; set for the problems that launch_gemm would
+    // split, whose shorter sums are the more precise ones
+    int pieces;
     // fault injection (tests of the failure path; 0 in normal use): the
     // split-K arrival wait expects split_extra arrivals beyond the splits
     // that exist, and gives up after split_wait_ns (0: kWaitLimitNs)
@@ -171,12 +172,26 @@ inline uint32_t gemm_b_box_rows(int bn) { return bn < 128 ? (uint32_t)bn : 128u;
 
 // 256-wide GEMM on CTA pairs (clusters of two, cta_group::2 MMAs of 256
 // rows): same parameters and epilogues as launch_gemm with bn = 256, K a
-// multiple of 128, no split K (p.ws null); tb in boxes of kGemmPairBBox rows
-// x 64 columns.  The
-// grid is min(max_pair_tiles, resident clusters) clusters.
-constexpr uint32_t kGemmPairBBox = 64;
-cudaError_t launch_gemm_pair(const CUtensorMap *ta, const CUtensorMap *tb, const GemmParams &p, int epi,
-                             int max_pair_tiles, cudaStream_t s);
+// multiple of 128, no workspace (p.ws null).  The grid is min(max_units,
+// resident clusters) clusters; 64-column units are the smallest the kernel
+// makes.
+// Operand maps: a stage's 128 K of an operand come with one TMA load, so a map
+// is a 3-D view [K / 64][rows][64] whose boxes hold two 64-column slices of
+// its rows: 128 rows of A; of B the 128, 64 or 32 rows that a CTA holds of a
+// 256-, 128- or 64-column unit.  (Loads of 64 columns x 64 rows, six per
+// stage instead of two: 25000 x 4096 x 1024 134.5 us against 124.5; ten per stage:
+// 143.)
+struct GemmPairB {
+    CUtensorMap rows[3];  // 128, 64 and 32 rows
+};
+bool make_tmap_pair(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, uint32_t box_rows);
+bool make_tmap_pair_b(GemmPairB *maps, const void *base, uint64_t rows, uint64_t K);
+// f3dc_gemm's rule: pairs for every shape they can compute.  At 1229 x 1024 x
+// 4096 they take 16.4 us against 29.9 us for the single-CTA kernel with split K,
+// at 1 x 1024 x 4096 14.1 us against 28.8 us.
+inline bool gemm_on_pairs(int N, int K) { return N % 256 == 0 && K % 128 == 0; }
+cudaError_t launch_gemm_pair(const CUtensorMap *ta, const GemmPairB *tb, const GemmParams &p, int epi, int max_units,
+                             cudaStream_t s);
 size_t gemm_smem_bytes(int bn);
 
 // Launches a kernel of this library with programmatic stream serialization

@@ -111,8 +111,8 @@ extern "C" f3dc_status f3dc_gemm_noalloc(const void *A, const void *B, const voi
     const int tiles = m_tiles * (N / bn);
     const int grid = gemm_grid(tiles, sms);
     const int splits = gemm_split_count(tiles, grid, K / 64, sms, true);
-    const bool pair = bn == 256 && K % 128 == 0 && splits == 1;
-    const size_t need = splits > 1 ? gemm_ws_bytes(bn, tiles * splits) : 0;
+    const bool pair = gemm_on_pairs(N, K);
+    const size_t need = !pair && splits > 1 ? gemm_ws_bytes(bn, tiles * splits) : 0;
     if (need > kPartialBytes)
         return fail(F3DC_ERR_INVALID_ARG, "this problem needs " + std::to_string(need) +
                                               " bytes of split-K scratch; the static scratch holds " +
@@ -123,8 +123,9 @@ extern "C" f3dc_status f3dc_gemm_noalloc(const void *A, const void *B, const voi
     if (e != cudaSuccess) return fail(F3DC_ERR_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
 
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, A, M, K, K, 128, 64) ||
-        !make_tmap_bf16(&tb, B, N, K, K, pair ? kGemmPairBBox : gemm_b_box_rows(bn), 64))
+    GemmPairB tbp;
+    if (!(pair ? make_tmap_pair(&ta, A, M, K, 128) && make_tmap_pair_b(&tbp, B, N, K)
+               : make_tmap_bf16(&ta, A, M, K, K, 128, 64) && make_tmap_bf16(&tb, B, N, K, K, gemm_b_box_rows(bn), 64)))
         return fail(F3DC_ERR_INVALID_ARG, "cuTensorMapEncodeTiled rejected A or B (alignment?)");
     GemmParams p;
     memset(&p, 0, sizeof(p));
@@ -140,8 +141,13 @@ extern "C" f3dc_status f3dc_gemm_noalloc(const void *A, const void *B, const voi
     const int epi = epilogue == F3DC_EPI_BIAS ? kEpiBias : (epilogue == F3DC_EPI_GELU ? kEpiGelu : kEpiResid);
     cudaStream_t s = (cudaStream_t)stream;
     if (pair) {
-        p.narrow_below = sms / 2;
-        e = launch_gemm_pair(&ta, &tb, p, epi, (m_tiles + 1) / 2 * (N / 128), s);
+        p.pieces = splits > 1;
+        e = launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s);
+        if (e != cudaSuccess) return fail(F3DC_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
+        return F3DC_OK;
+    }
+    if (splits == 1) {
+        e = launch_gemm(&ta, &tb, p, epi, bn, tiles < sms ? tiles : sms, s);
         if (e != cudaSuccess) return fail(F3DC_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
         return F3DC_OK;
     }

@@ -107,3 +107,33 @@ def test_gemm_split_k_repeat_is_deterministic(orc):
         outs.append(x)
     torch.cuda.synchronize()
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+@pytest.mark.parametrize("M,N,K", [(63, 1024, 2048), (64, 1024, 2048), (257, 256, 128), (1229, 1024, 4096),
+                                   (1229, 4096, 128), (1300, 4096, 256), (2400, 1024, 2048), (4096, 4096, 128),
+                                   (5000, 1024, 384)])
+@pytest.mark.parametrize("epi", [f3dc.EPI_BIAS, f3dc.EPI_RESID])
+def test_gemm_pair_units(M, N, K, epi):
+    # the CTA-pair kernel's work units, every element against 64 bits: last
+    # waves of 64-, 128- and 256-column units (63 and 64 rows lie on either
+    # side of the row limit of the narrowest), full waves with a rest (80, 96,
+    # 256 and 80 tiles on 76 clusters), odd row tiles, and sums in several
+    # accumulators (K >= 2048 on few tiles; 2400 rows: two of 256 columns)
+    A, Bw, bias, gate, _ = _inputs(M, N, K, M + N + K + epi)
+    Ad, Bd, bd, gd = dev_bf16(A), dev_bf16(Bw), dev_bf16(bias), dev_f32(gate)
+    y = Ad.double() @ Bd.double().T + bd.double()
+    if epi == f3dc.EPI_BIAS:
+        out = torch.full((M, N), 7.0, dtype=torch.bfloat16, device="cuda")
+        f3dc.gemm(Ad, Bd, bd, None, out, M, N, K, epi)
+        # one bf16 rounding (2^-9 of the value) and the fp32 sum
+        assert torch.all((out.double() - y).abs() <= 2.0 ** -8 * y.abs() + 1e-4)
+    else:
+        x0 = dev_f32(np.random.default_rng(M).standard_normal((M, N)).astype(np.float32))
+        out = x0.clone()
+        f3dc.gemm(Ad, Bd, bd, gd, out, M, N, K, epi)
+        ref = x0.double() + gd.double() * y
+        # the tensor core's sums are off by at most ~8e-10 K relative (truncation),
+        # with pieces of at most 1024 for K > 2048; the rest rounds at 2^-24
+        assert ((out.double() - ref).norm() / ref.norm()).item() < 2e-6
+        assert (out.double() - ref).abs().max().item() < 1e-4
+    assert f3dc.gemm_status() == 0
