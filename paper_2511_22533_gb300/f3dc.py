@@ -68,6 +68,8 @@ def library_path() -> str:
 def lib():
     """Loads libf3dc.so (building it first if the sources are newer)."""
     global _lib
+    if _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build()
@@ -125,17 +127,27 @@ def _check(status, handle=None):
         raise F3dcError(status, msg.decode() if msg else "")
 
 
+# Pointer arguments are plain integers (the functions' argtypes convert them):
+# a small call is bound by this marshalling, not by its kernel.
 def _ptr(t):
-    if t is None:
-        return None
-    return C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_current_raw_stream = None
 
 
 def _stream(stream):
+    """The given stream, or the current one of the current device (its handle
+    alone: torch.cuda.current_stream() builds a Stream object per call)."""
+    global _current_raw_stream
     if stream is not None:
-        return C.c_void_p(stream)
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return stream
+    if _current_raw_stream is None:
+        import torch
+        torch.cuda.init()
+        get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        _current_raw_stream = lambda: get_stream(get_device())  # noqa: E731
+    return _current_raw_stream()
 
 
 def _np_ptr(a, typ):
