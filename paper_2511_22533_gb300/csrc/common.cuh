@@ -547,6 +547,12 @@ F3DC_DEV f32x2 fmul2(f32x2 a, f32x2 b)
     return r;
 }
 
+// A product that must round on its own before it is added: the compiler makes
+// one FMA of mul.rn.f32x2 and add.rn.f32x2 (with -fmad=false too), unlike of the
+// scalar __fmul_rn and __fadd_rn.  An FMA with an addend of -0.0 is the product
+// alone, and the compiler cannot see the addend: it comes from a kernel argument.
+F3DC_DEV f32x2 fmul2_alone(f32x2 a, f32x2 b, float neg_zero) { return ffma2(a, b, {neg_zero, neg_zero}); }
+
 F3DC_DEV float gelu_tanh(float x)
 {
     const float k0 = 0.7978845608028654f;  // sqrt(2/pi)

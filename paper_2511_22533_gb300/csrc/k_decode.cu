@@ -18,9 +18,10 @@
 // so a thread computes the two (hidden layer) or four (last layer) of a cell,
 // with channel-last activations read 16 bytes at a time.  One decode of eight
 // 16^3 samples: 517 us with one output voxel per thread and channel-major
-// activations, 141 us now (one sample: 108 -> 34 us).  The hidden layers run at
+// activations, 154 us now (one sample: 108 -> 37 us).  The hidden layers run at
 // 200 registers and two blocks per SM: with 128 (four blocks) the three source
-// voxels spill, and the decode takes 224 us.
+// voxels spill, and the decode took 224 us against 141 (before each product was
+// made to round on its own, see fmul2_alone).
 #include "common.cuh"
 #include "kernels.h"
 
@@ -48,7 +49,7 @@ F3DC_DEV void load_voxel(const float *p, float (&v)[C])
 // UP voxels along x that share source column sx.
 template <int CIN, int COUT, int UP>
 __global__ void __launch_bounds__(kDecThreads, 2) k_conv3d(const float *in, int din, const uint16_t *w,
-                                                       const uint16_t *bias, float *out, int B)
+                                                       const uint16_t *bias, float *out, int B, float neg_zero)
 {
     constexpr int G = COUT / 8;
     // [tap][ci][co], taps 16 bytes further apart: a warp fills consecutive taps
@@ -94,10 +95,10 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_conv3d(const float *in, int 
             for (int ci = 0; ci < CIN; ++ci) {
                 const float4 w0 = wk[ci * (COUT / 4)], w1 = wk[ci * (COUT / 4) + 1];
                 const f32x2 x = {v[ci], v[ci]};
-                a[0] = fadd2(a[0], fmul2(x, {w0.x, w0.y}));
-                a[1] = fadd2(a[1], fmul2(x, {w0.z, w0.w}));
-                a[2] = fadd2(a[2], fmul2(x, {w1.x, w1.y}));
-                a[3] = fadd2(a[3], fmul2(x, {w1.z, w1.w}));
+                a[0] = fadd2(a[0], fmul2_alone(x, {w0.x, w0.y}, neg_zero));
+                a[1] = fadd2(a[1], fmul2_alone(x, {w0.z, w0.w}, neg_zero));
+                a[2] = fadd2(a[2], fmul2_alone(x, {w1.x, w1.y}, neg_zero));
+                a[3] = fadd2(a[3], fmul2_alone(x, {w1.z, w1.w}, neg_zero));
             }
         };
         if (UP == 1) {
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) k_conv3d(const float *in, int 
 // stored ones into dyn[b] instead of storing.
 __global__ void __launch_bounds__(kDecThreads) k_conv3d_occ(const float *in, int din, const uint16_t *w,
                                                            const uint16_t *bias, uint32_t *bits, int compare,
-                                                           int64_t *dyn, int B)
+                                                           int64_t *dyn, int B, float neg_zero)
 {
     constexpr int CIN = 8;
     __shared__ float2 sw[27][CIN];  // each weight twice, for the paired instructions
@@ -180,7 +181,8 @@ __global__ void __launch_bounds__(kDecThreads) k_conv3d_occ(const float *in, int
 #pragma unroll
                     for (int ci = 0; ci < CIN; ++ci) {
                         const float2 wv = sw[9 * kz + 3 * ky + kx][ci];
-                        const f32x2 n = fadd2(acc[j], fmul2({s[jr][c0][ci], s[jr][c1][ci]}, {wv.x, wv.y}));
+                        const f32x2 n =
+                            fadd2(acc[j], fmul2_alone({s[jr][c0][ci], s[jr][c1][ci]}, {wv.x, wv.y}, neg_zero));
                         // taps outside the grid are skipped
                         acc[j].x = kx == 0 && !lo ? acc[j].x : n.x;
                         acc[j].y = kx == 2 && !hi ? acc[j].y : n.y;
@@ -225,13 +227,13 @@ cudaError_t launch_decode_conv(const DecodeArgs &a, cudaStream_t s)
     float *x1 = a.scratch, *x2 = a.scratch + B * 16 * N;
     // C -> 16 at D^3 from the token-major latents S [B, N, 8]
     launch_k(k_conv3d<kChannels, 16, 1>, dim3(dec_grid(B * N * 2)), dim3(kDecThreads), 0, s, a.S, D, a.w1, a.b1, x1,
-             a.B);
+             a.B, -0.0f);
     // 16 -> 8 at (2D)^3
     launch_k(k_conv3d<16, 8, 2>, dim3(dec_grid(B * 4 * N)), dim3(kDecThreads), 0, s, (const float *)x1, D, a.w2, a.b2,
-             x2, a.B);
+             x2, a.B, -0.0f);
     // 8 -> 1 at (4D)^3, to bits
     launch_k(k_conv3d_occ, dim3(dec_grid(B * 16 * N)), dim3(kDecThreads), 0, s, (const float *)x2, 2 * D, a.w3, a.b3,
-             a.bits, a.compare, a.dyn, a.B);
+             a.bits, a.compare, a.dyn, a.B, -0.0f);
     return cudaGetLastError();
 }
 

@@ -7,7 +7,7 @@ import pytest
 import torch
 
 from gpu_helpers import assert_clean, dev_f32, dev_i32, dev_u16, handle_for
-from paper_2511_22533_gb300 import synth
+from paper_2511_22533_gb300 import f3dc, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -44,6 +44,35 @@ def test_anchor_step_dynamic_voxels_exact(orc, shape):
 def test_anchor_step_dynamic_voxels_exact_on_odd_rows(orc, grid):
     # grid rows that do not fill a warp (and 20^3: a last block that is not full)
     test_anchor_step_dynamic_voxels_exact(orc, synth.ModelShape(grid, 8, 128, 1, 4, 4, 64, 128, 8, 64))
+
+
+@pytest.mark.parametrize("layer", [1, 2, 3])
+def test_decoder_rounds_every_product(orc, layer):
+    # 0.6666667 * 1.5 - 1 is 0 when the product rounds on its own (to 1) and
+    # 2^-25 when it does not: with that in one layer and the others passing
+    # their centre through, the grid before the step is empty or full.  Every
+    # token is cached with a velocity that leaves an empty grid after the step.
+    shape = synth.ModelShape(8, 8, 128, 1, 4, 4, 64, 128, 8, 64)
+    N, k = shape.tokens, 3
+    blob = synth.weights_blob(shape, 0)
+    for n, (co, ci) in enumerate([(16, 8), (8, 16), (1, 8)], 1):
+        w = np.zeros((co, ci, 27), np.float32)
+        w[:, 0, 13] = 1.5 if n == layer else 1.0
+        synth.set_weight(blob, shape, f"dc{n}_w", -1, w.reshape(co, ci * 27))
+        synth.set_weight(blob, shape, f"dc{n}_b", -1, np.full(co, -1.0 if n == layer else 0.0, np.float32))
+    h = f3dc.Handle(f3dc.config_for(shape, 1, decoder=1), dev_u16(blob))
+    h.set_cond(dev_u16(synth.cond_tokens(shape, 1, 2)), 1)
+    S = np.full((1, N, 8), np.float32(2.0) / np.float32(3.0), np.float32)
+    ring = np.zeros((3, 1, N, 8), np.uint16)
+    ring[(k - 1) % 3] = synth.f32_to_bf16_bits(np.full((1, N, 8), 64.0, np.float32))
+    S_d, dyn = dev_f32(S), torch.zeros(1, dtype=torch.int64, device="cuda")
+    h.step(k, 1, S_d, dev_u16(ring), dev_i32([N]), dyn_voxels=dyn)
+    torch.cuda.synchronize()
+    assert_clean(h)
+    m = orc.Model(shape, blob)
+    assert not np.any(m.decode_conv(S_d.cpu().numpy()[0])) and not np.any(m.decode_conv(S[0]))
+    assert dyn.item() == 0
+    h.close()
 
 
 def test_sampler_sigma_with_conv_decoder(orc):
