@@ -13,12 +13,26 @@
 // order-preserving 32-bit key per token (in place of V), and a 4 x 8-bit
 // radix select finds the c-th smallest key of the sample: every CTA counts
 // its keys into a 256-bin histogram, the cluster sums the eight histograms
-// bin by bin (each CTA redundantly, so all take the same digit).  Finally
+// bin by bin (each CTA redundantly, so all take the same digit), and ends at the first digit whose keys are all
+// cached.  Finally
 // each CTA caches its keys below the threshold plus the lowest-index ties
 // and compacts its active tokens in ascending order, starting from the
 // counts of the lower-ranked CTAs.  With a third history slot (SSC with
 // three predictions) the acceleration term is the second difference of the
 // velocity and each token reads 48 B.
+//
+// What bounds it: at large batches the load of all samples at once, then the
+// passes over shared memory (batch 64 on the 32^3 grid, 73 MB: 40.7 us with
+// scalar sums and divisions, four full radix passes and outputs written one at
+// a time; 32.2 us = 2.3 TB/s now).  For one sample the chain of cluster barriers
+// (16^3, one after another: 9.9 -> 7.9 us per call; the search ends at the first
+// digit whose keys are all cached, usually the third).  Device time of the parts
+// at batch 64: paired norms, shared reciprocals and wide outputs 39.0 -> 30.9 us,
+// the early end 29.3, the keys' spacing and one histogram after the first pass
+// 28.4.  Measured slower: 3 x 10-bit digits (45.7 us: every CTA reads eight
+// histograms of 1024 bins per pass).
+#include <atomic>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -33,26 +47,27 @@ constexpr int kSelMaxTokens = 49152;  // per sample: 8 B of shared memory per to
 constexpr int kSelUnroll = 4;         // tokens of a thread whose loads are in flight together
 
 // V = |v1|, A = |v1 - v2| (Sec. 4.1), or with v3 the second difference
-// |(v1 - v2) - (v2 - v3)|, each channel term in that fp32 order.
-F3DC_DEV void token_va(const uint4 &p, const uint4 &q, const uint4 &r, bool third, float &V, float &A)
+// |(v1 - v2) - (v2 - v3)|, each channel term in that fp32 order.  The two sums
+// of squares run side by side in paired instructions.
+template <bool kThird>
+F3DC_DEV void token_va(const uint4 &p, const uint4 &q, const uint4 &r, float neg_zero, float &V, float &A)
 {
     const uint32_t pw[4] = {p.x, p.y, p.z, p.w};
     const uint32_t qw[4] = {q.x, q.y, q.z, q.w};
     const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-    float sv = 0.0f, sa = 0.0f;
+    f32x2 s = {0.0f, 0.0f};
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        const uint32_t pu = (pw[c >> 1] >> ((c & 1) * 16)) & 0xFFFFu;
-        const uint32_t qu = (qw[c >> 1] >> ((c & 1) * 16)) & 0xFFFFu;
-        const float x = bf16_bits_to_f32(pu);
-        const float y = bf16_bits_to_f32(qu);
+        auto at = [&](const uint32_t(&w)[4]) {
+            return __uint_as_float(c & 1 ? w[c >> 1] & 0xFFFF0000u : w[c >> 1] << 16);
+        };
+        const float x = at(pw), y = at(qw);
         float d = __fsub_rn(x, y);
-        if (third) d = __fsub_rn(d, __fsub_rn(y, bf16_bits_to_f32((rw[c >> 1] >> ((c & 1) * 16)) & 0xFFFFu)));
-        sv = __fadd_rn(sv, __fmul_rn(x, x));
-        sa = __fadd_rn(sa, __fmul_rn(d, d));
+        if (kThird) d = __fsub_rn(d, __fsub_rn(y, at(rw)));
+        s = fadd2(s, fmul2_alone({x, d}, {x, d}, neg_zero));
     }
-    V = __fsqrt_rn(sv);
-    A = __fsqrt_rn(sa);
+    V = __fsqrt_rn(s.x);
+    A = __fsqrt_rn(s.y);
 }
 
 // min-max normalisation; NaN stays NaN, a degenerate range gives 0.
@@ -63,14 +78,32 @@ F3DC_DEV float norm1(float x, float mn, float mx)
     return __fdiv_rn(__fsub_rn(x, mn), __fsub_rn(mx, mn));
 }
 
-// Order-preserving key: equal floats (including -0 / +0) give equal keys,
-// every NaN gives the largest key (never cached before a number).
+// The same division for both norms of a token when both ranges d lie in
+// [2^-98, 2^20] (`inv` = 1 / d, correctly rounded): n inv, then twice a
+// residual and its correction (Markstein, "Computation of elementary functions
+// on the IBM RISC System/6000 processor", 1990): with a correctly rounded
+// reciprocal and a quotient within one unit, RN(q + RN(n - q d) inv) is the
+// correctly rounded quotient.  Nothing underflows on the way: a norm is 0 or at
+// least 2^-74.5 (the root of a bf16 square's fp32 sum), so n is 0 or at least
+// 2^-98, the quotient at least 2^-118 and the residual a multiple of 2^-145.
+F3DC_DEV f32x2 div_by_range(f32x2 n, f32x2 d, f32x2 inv)
+{
+    const f32x2 nd = {-d.x, -d.y};
+    f32x2 q = fmul2(n, inv);
+    q = ffma2(ffma2(q, nd, n), inv, q);
+    return ffma2(ffma2(q, nd, n), inv, q);
+}
+
+// Order-preserving key of a score, 0 <= score < 1 + 2^-20: its bits, with the
+// distances above 2^-6 stretched 64 times, so that a binade there covers 32
+// values of the first radix digit (as the bits stand it would cover one half)
+// and the largest key stays below 2^32; every NaN gives the largest key (never
+// cached before a number).
 F3DC_DEV uint32_t score_key(float s)
 {
-    if (isnan(s)) return 0xFFFFFFFFu;
-    if (s == 0.0f) s = 0.0f;
+    constexpr uint32_t kKnee = 0x3C800000u;  // 2^-6
     const uint32_t u = __float_as_uint(s);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return isnan(s) ? 0xFFFFFFFFu : (u < kKnee ? u : kKnee + ((u - kKnee) << 6));
 }
 
 F3DC_DEV int pad_tile(int a) { return (a + kTileRows - 1) / kTileRows * kTileRows; }
@@ -163,11 +196,13 @@ F3DC_DEV uint32_t block_scan(uint32_t v, uint32_t *wsum, uint32_t *total)
     return before + incl;
 }
 
-__global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4) k_ssc_select(const SelectArgs a)
+template <bool kThird>
+__global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
+    k_ssc_select(const SelectArgs a, float neg_zero)
 {
     griddep_launch();
     griddep_wait();
-    extern __shared__ float sva[];            // V, A of this CTA's tokens; the key later replaces V
+    extern __shared__ __align__(16) float sva[];  // V, A of this CTA's tokens; the key later replaces V
     __shared__ uint32_t whist[kSelWarps / 2][256];  // one histogram per warp pair
     // this CTA's histogram of the current radix pass (read by the cluster);
     // two buffers: pass p + 1 writes the buffer that pass p - 1's readers
@@ -178,7 +213,7 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
     __shared__ float red[4][kSelWarps];
     __shared__ float gmm[4];
     __shared__ uint32_t wsum[kSelWarps];
-    __shared__ uint32_t s_digit, s_rank;
+    __shared__ uint32_t s_digit, s_rank, s_ties;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t rk = cluster_rank();
@@ -215,7 +250,7 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
     // ---- V and A of this CTA's tokens, min / max (NaN never wins a comparison)
     const uint4 *g1 = reinterpret_cast<const uint4 *>(a.v1) + base + lo;
     const uint4 *g2 = reinterpret_cast<const uint4 *>(a.v2) + base + lo;
-    const uint4 *g3 = a.v3 ? reinterpret_cast<const uint4 *>(a.v3) + base + lo : nullptr;
+    const uint4 *g3 = kThird ? reinterpret_cast<const uint4 *>(a.v3) + base + lo : nullptr;
     float mnV = INFINITY, mxV = -INFINITY, mnA = INFINITY, mxA = -INFINITY;
     for (int i0 = tid; i0 < nl; i0 += kSelUnroll * kSelThreads) {
         uint4 p[kSelUnroll], q[kSelUnroll], r[kSelUnroll];
@@ -225,7 +260,7 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
             if (i < nl) {
                 p[u] = __ldg(g1 + i);
                 q[u] = __ldg(g2 + i);
-                r[u] = g3 ? __ldg(g3 + i) : make_uint4(0, 0, 0, 0);
+                r[u] = kThird ? __ldg(g3 + i) : make_uint4(0, 0, 0, 0);
             }
         }
 #pragma unroll
@@ -233,13 +268,13 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
             const int i = i0 + u * kSelThreads;
             if (i < nl) {
                 float V, A;
-                token_va(p[u], q[u], r[u], g3 != nullptr, V, A);
+                token_va<kThird>(p[u], q[u], r[u], neg_zero, V, A);
                 sV[i] = V;
                 sA[i] = A;
-                if (V < mnV) mnV = V;
-                if (V > mxV) mxV = V;
-                if (A < mnA) mnA = A;
-                if (A > mxA) mxA = A;
+                mnV = fminf(mnV, V);
+                mxV = fmaxf(mxV, V);
+                mnA = fminf(mnA, A);
+                mxA = fmaxf(mxA, A);
             }
         }
     }
@@ -280,14 +315,27 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
     mxA = gmm[3];
 
     // ---- C_i = w_a norm(A_i) + w_v norm(V_i) -> ordered keys, and the
-    // histogram of their top byte (the first radix pass)
+    // histogram of their top digit (the first radix pass)
     for (int q = tid; q < kSelWarps / 2 * 256; q += kSelThreads) (&whist[0][0])[q] = 0;
     __syncthreads();
-    for (int i = tid; i < nl; i += kSelThreads) {
-        const float sc = __fadd_rn(__fmul_rn(a.wa, norm1(sA[i], mnA, mxA)), __fmul_rn(a.wv, norm1(sV[i], mnV, mxV)));
-        const uint32_t k = score_key(sc);
-        keys[i] = k;
-        atomicAdd(&whist[warp >> 1][k >> 24], 1u);
+    const f32x2 d = {__fsub_rn(mxV, mnV), __fsub_rn(mxA, mnA)};
+    auto plain = [](float x) { return x >= 0x1p-98f && x <= 0x1p20f; };
+    if (plain(d.x) && plain(d.y)) {
+        const f32x2 inv = {__frcp_rn(d.x), __frcp_rn(d.y)};
+        for (int i = tid; i < nl; i += kSelThreads) {
+            const f32x2 q = div_by_range({__fsub_rn(sV[i], mnV), __fsub_rn(sA[i], mnA)}, d, inv);
+            const uint32_t k = score_key(__fadd_rn(__fmul_rn(a.wa, q.y), __fmul_rn(a.wv, q.x)));
+            keys[i] = k;
+            atomicAdd(&whist[warp >> 1][k >> 24], 1u);
+        }
+    } else {
+        for (int i = tid; i < nl; i += kSelThreads) {
+            const float sc =
+                __fadd_rn(__fmul_rn(a.wa, norm1(sA[i], mnA, mxA)), __fmul_rn(a.wv, norm1(sV[i], mnV, mxV)));
+            const uint32_t k = score_key(sc);
+            keys[i] = k;
+            atomicAdd(&whist[warp >> 1][k >> 24], 1u);
+        }
     }
     __syncthreads();
 
@@ -301,17 +349,19 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
     for (int pass = 0; pass < 4; ++pass) {
         const int shift = 24 - 8 * pass;
         if (pass > 0) {
-            for (int q = tid; q < kSelWarps / 2 * 256; q += kSelThreads) (&whist[0][0])[q] = 0;
+            whist[0][tid] = 0;  // few keys are left: one histogram
             __syncthreads();
             for (int i = tid; i < nl; i += kSelThreads) {
                 const uint32_t k = keys[i];
-                if ((k & hi_mask) == prefix) atomicAdd(&whist[warp >> 1][(k >> shift) & 255u], 1u);
+                if ((k & hi_mask) == prefix) atomicAdd(&whist[0][(k >> shift) & 255u], 1u);
             }
             __syncthreads();
         }
-        uint32_t v = 0;
+        uint32_t v = whist[0][tid];
+        if (pass == 0) {
 #pragma unroll
-        for (int w = 0; w < kSelWarps / 2; ++w) v += whist[w][tid];
+            for (int w = 1; w < kSelWarps / 2; ++w) v += whist[w][tid];
+        }
         hist[pass & 1][tid] = v;
         cluster_sync();  // every CTA's histogram of this pass is complete
         uint32_t tot = 0;
@@ -323,22 +373,26 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
         if (excl < rank && rank <= incl) {
             s_digit = (uint32_t)tid;
             s_rank = rank - excl;
+            s_ties = tot;
         }
         __syncthreads();
         prefix |= s_digit << shift;
         hi_mask |= 255u << shift;
         rank = s_rank;
-        __syncthreads();  // s_digit / s_rank are rewritten by the next pass
+        const uint32_t ties = s_ties;
+        __syncthreads();  // rewritten by the next pass
+        if (ties == rank) break;  // every key with these digits is cached: the rest cannot matter
     }
-    const uint32_t thr = prefix;  // keys below thr are cached, plus the first `rank` ties of the sample
+    // keys below thr in the digits found are cached, plus the first `rank` ties of the sample
+    const uint32_t thr = prefix;
 
     // ---- this CTA's keys below / at the threshold; the lower-ranked CTAs'
     // counts give the sample-wide counts before this CTA's first token
     uint32_t nlt = 0, neq = 0;
     for (int i = tid; i < nl; i += kSelThreads) {
         const uint32_t k = keys[i];
-        nlt += k < thr;
-        neq += k == thr;
+        nlt += (k & hi_mask) < thr;
+        neq += (k & hi_mask) == thr;
     }
     uint32_t all_lt, all_eq;
     block_scan(nlt, wsum, &all_lt);
@@ -388,48 +442,51 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
     // thread takes four consecutive tokens per round of 1024.
     for (int j0 = 0; j0 < nl; j0 += 4 * kSelThreads) {
         const int j = j0 + 4 * tid;
-        uint32_t k[4];
-        if (j + 3 < nl) {
-            const uint4 kk = *reinterpret_cast<const uint4 *>(keys + j);
-            k[0] = kk.x;
-            k[1] = kk.y;
-            k[2] = kk.z;
-            k[3] = kk.w;
-        } else {
-#pragma unroll
-            for (int r2 = 0; r2 < 4; ++r2) k[r2] = j + r2 < nl ? keys[j + r2] : 0u;
-        }
+        // nl is a multiple of 4: a thread's four tokens exist or none does
         uint32_t ltb = 0, eqb = 0;
-#pragma unroll
-        for (int r2 = 0; r2 < 4; ++r2) {
-            if (j + r2 < nl) {
-                ltb |= (uint32_t)(k[r2] < thr) << r2;
-                eqb |= (uint32_t)(k[r2] == thr) << r2;
-            }
+        if (j < nl) {
+            uint4 kk = *reinterpret_cast<const uint4 *>(keys + j);
+            kk = make_uint4(kk.x & hi_mask, kk.y & hi_mask, kk.z & hi_mask, kk.w & hi_mask);
+            ltb = (kk.x < thr ? 1u : 0u) | (kk.y < thr ? 2u : 0u) | (kk.z < thr ? 4u : 0u) | (kk.w < thr ? 8u : 0u);
+            eqb = (kk.x == thr ? 1u : 0u) | (kk.y == thr ? 2u : 0u) | (kk.z == thr ? 4u : 0u) | (kk.w == thr ? 8u : 0u);
         }
         const uint32_t cnt4 = (uint32_t)__popc(ltb) | ((uint32_t)__popc(eqb) << 16);
         uint32_t tot;
         const uint32_t pre = block_scan(cnt4, wsum, &tot) - cnt4;
-        uint32_t plt = run_lt + (pre & 0xFFFFu), peq = run_eq + (pre >> 16);
+        if (j < nl) {
+            uint32_t plt = run_lt + (pre & 0xFFFFu), peq = run_eq + (pre >> 16);
+            const int i0 = lo + j;
+            uint32_t mask4 = 0;
+            int row[4];
 #pragma unroll
-        for (int r2 = 0; r2 < 4; ++r2) {
-            if (j + r2 >= nl) break;
-            const int i = lo + j + r2;
-            const bool lt = (ltb >> r2) & 1u, eq = (eqb >> r2) & 1u;
-            const bool cached = lt || (eq && peq < rank);
-            if (a.mask) a.mask[base + i] = cached ? 1 : 0;
-            if (!cached) {
-                const uint32_t pos = (uint32_t)i - plt - min(peq, rank);
-                if (pos >= (uint32_t)na) raise_error(a.err, kDevBadPlan);
-                else {
-                    a.active_idx[base + pos] = i;
-                    if (a.row_of_token) a.row_of_token[base + i] = off + (int)pos;
+            for (int r2 = 0; r2 < 4; ++r2) {
+                const uint32_t lt = (ltb >> r2) & 1u, eq = (eqb >> r2) & 1u;
+                const bool cached = lt || (eq && peq < rank);
+                row[r2] = -1;
+                if (cached) {
+                    mask4 |= 1u << (8 * r2);
+                } else {
+                    const uint32_t pos = (uint32_t)(i0 + r2) - plt - min(peq, rank);
+                    if (pos >= (uint32_t)na) {
+                        raise_error(a.err, kDevBadPlan);
+                    } else {
+                        a.active_idx[base + pos] = i0 + r2;
+                        row[r2] = off + (int)pos;
+                    }
                 }
-            } else if (a.row_of_token) {
-                a.row_of_token[base + i] = -1;
+                plt += lt;
+                peq += eq;
             }
-            plt += lt;
-            peq += eq;
+            if (a.mask) {
+                uint8_t *m = a.mask + base + i0;
+                if (((uintptr_t)a.mask & 3) == 0) {
+                    *reinterpret_cast<uint32_t *>(m) = mask4;
+                } else {  // the caller's mask may start anywhere
+#pragma unroll
+                    for (int r2 = 0; r2 < 4; ++r2) m[r2] = (uint8_t)((mask4 >> (8 * r2)) & 1u);
+                }
+            }
+            if (a.row_of_token) *reinterpret_cast<int4 *>(a.row_of_token + base + i0) = make_int4(row[0], row[1], row[2], row[3]);
         }
         run_lt += tot & 0xFFFFu;
         run_eq += tot >> 16;
@@ -467,6 +524,25 @@ __global__ void k_plan_from_counts(const int32_t *n_active, int B, int N, Plan *
     }
 }
 
+template <bool kThird>
+cudaError_t launch_select(const SelectArgs &a, size_t smem, cudaStream_t s)
+{
+    // the shared-memory attribute is per device: set it on each device's first launch
+    static std::atomic<uint64_t> attr_devices{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (!(attr_devices.load(std::memory_order_acquire) & bit)) {
+        e = cudaFuncSetAttribute(k_ssc_select<kThird>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSelMaxTokens / kSelCS * 2 * (int)sizeof(float));
+        if (e != cudaSuccess) return e;
+        attr_devices.fetch_or(bit, std::memory_order_acq_rel);
+    }
+    launch_k(k_ssc_select<kThird>, dim3(a.B * kSelCS), dim3(kSelThreads), smem, s, a, -0.0f);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 int ssc_select_max_tokens() { return kSelMaxTokens; }
@@ -478,12 +554,7 @@ cudaError_t launch_ssc_select(const SelectArgs &a, cudaStream_t s)
         return cudaErrorInvalidValue;
     // V and A of a CTA's tokens (the key later replaces V)
     const size_t smem = (size_t)(a.N / kSelCS) * 2 * sizeof(float);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_ssc_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    launch_k(k_ssc_select, dim3(a.B * kSelCS), dim3(kSelThreads), smem, s, a);
-    return cudaGetLastError();
+    return a.v3 ? launch_select<true>(a, smem, s) : launch_select<false>(a, smem, s);
 }
 
 cudaError_t launch_plan_from_counts(const int32_t *n_active, const int32_t *active_idx, int B, int N,

@@ -116,3 +116,51 @@ def test_selection_batch64_32cubed(orc):
     idx, na, mask = _run(h, hist, qs)
     _check(orc, hist, qs, idx, na, mask)
     h.close()
+
+
+@pytest.mark.parametrize("log2_scale", [25, -40, -70])
+def test_selection_at_scaled_velocities(orc, h16, log2_scale):
+    # the shared-reciprocal division serves ranges in [2^-98, 2^20]: above it
+    # (2^25) the general one runs; at 2^-70 the squares' sums are subnormal
+    hist = synth.velocity_history(16, 8, 2, seed=11)
+    scaled = synth.f32_to_bf16_bits(np.ldexp(synth.bf16_bits_to_f32(hist), log2_scale))
+    qs = np.array([1500, 3001], np.int32)
+    idx, na, mask = _run(h16, scaled, qs)
+    _check(orc, scaled, qs, idx, na, mask)
+
+
+def test_selection_mask_at_any_address(orc, h16):
+    hist = synth.velocity_history(16, 8, 1, seed=12)
+    N = 4096
+    idx = torch.full((1, N), -1, dtype=torch.int32, device="cuda")
+    na = torch.zeros(1, dtype=torch.int32, device="cuda")
+    buf = torch.full((N + 8,), 9, dtype=torch.uint8, device="cuda")
+    v1, v2 = dev_u16(hist[2]), dev_u16(hist[1])
+    h16.ssc_select(v1, v2, 1, dev_i32([1234]), idx, na, buf[3:])
+    torch.cuda.synchronize()
+    got = buf.cpu().numpy()
+    assert np.all(got[:3] == 9) and np.all(got[3 + N:] == 9)
+    _check(orc, hist, np.array([1234]), idx.cpu().numpy(), na.cpu().numpy(), got[None, 3:3 + N])
+
+
+@pytest.mark.parametrize("case", ["one_digit", "ties_across_ctas", "both_sides_of_the_knee"])
+def test_selection_where_the_radix_search_ends(orc, h16, case):
+    # the search ends at the first digit whose keys are all cached: after one
+    # pass, after all four (ties that must be broken by index), and with scores
+    # on both sides of 2^-6, where the keys' spacing changes
+    N = 4096
+    v = np.zeros((3, 1, N, 8), np.float32)
+    if case == "one_digit":
+        v[2, 0, :, 0] = np.where(np.arange(N) % 3 == 0, 1.0, 2.0)
+        q = np.count_nonzero(np.arange(N) % 3 == 0)
+    elif case == "ties_across_ctas":
+        v[2, 0, :, 0] = np.where(np.arange(N) % 5 == 0, 1.0, 2.0)
+        v[2, 0, 7, 0] = 0.0
+        q = 1 + 300
+    else:
+        v[2, 0, :, 0] = np.exp2(np.random.default_rng(3).uniform(-14, 0, N))
+        q = 2500
+    hist = synth.f32_to_bf16_bits(v)
+    qs = np.array([q], np.int32)
+    idx, na, mask = _run(h16, hist, qs)
+    _check(orc, hist, qs, idx, na, mask)
