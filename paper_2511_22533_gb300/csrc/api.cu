@@ -281,7 +281,7 @@ struct f3dc_handle {
     bf16 *h = nullptr, *qkv = nullptr, *att = nullptr, *qc = nullptr, *u = nullptr, *ckv = nullptr;
     uint16_t *ring = nullptr;
     Plan *plan = nullptr;
-    int32_t *tile_sample = nullptr, *active_idx = nullptr, *row_of_token = nullptr, *n_active = nullptr;
+    int32_t *tile_sample = nullptr, *pair_tiles = nullptr, *active_idx = nullptr, *row_of_token = nullptr, *n_active = nullptr;
     uint8_t *mask = nullptr;
     int32_t *quota_dev = nullptr;
     int64_t *dyn = nullptr;
@@ -496,8 +496,10 @@ cudaError_t run_attention(f3dc_handle *h, int mode, const CUtensorMap &tq, const
     p.mode = mode;
     p.n_tiles_dev = &h->plan->n_tiles;
     p.tile_sample = h->tile_sample;
+    p.pair_tiles = h->pair_tiles;
     p.plan = h->plan;
     p.nk_fixed = h->Nc;
+    p.q_rows = INT32_MAX;
     p.kv_null_from = mode == 1 ? h->cfg_B_now : 0;
     p.kv_null_sample = h->cfg.max_batch;
     p.kv_prefetch_rows = mode == 1 ? h->cond_B * h->Nc : 0;  // the condition's K / V
@@ -505,11 +507,11 @@ cudaError_t run_attention(f3dc_handle *h, int mode, const CUtensorMap &tq, const
     p.ldo = h->W;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)h->dh));
     p.err = h->dev_err;
-    // work items: (pair of query tiles, head)
     // persistent CTAs, one per work item up to one per SM: (query tile, head)
     // items for the one-tile kernel, (pair of query tiles, head) otherwise
     const bool one = h->attn_one_now;
-    const int items = one ? h->max_tiles * h->H : (h->max_tiles + 1) / 2 * h->H;
+    const int per_sample = (h->N + kTileRows - 1) / kTileRows;  // tiles; pairs are within a sample
+    const int items = (one ? h->max_tiles : h->max_tiles / per_sample * ((per_sample + 1) / 2)) * h->H;
     const int grid = items < h->num_sms ? items : h->num_sms;
     return one ? launch_attention_one(&tq, &tkv, &tkv, p, grid, s) : launch_attention(&tq, &tkv, &tkv, p, grid, s);
 }
@@ -696,7 +698,7 @@ bool build_maps(f3dc_handle *h)
 void free_handle(f3dc_handle *h)
 {
     void *ptrs[] = {h->wblob, h->mod_w, h->mod_b, h->pos, h->x, h->v_active, h->freq, h->h1, h->temb, h->mod,
-                    h->h, h->qkv, h->att, h->qc, h->u, h->ckv, h->ring, h->plan, h->tile_sample, h->active_idx,
+                    h->h, h->qkv, h->att, h->qc, h->u, h->ckv, h->ring, h->plan, h->tile_sample, h->pair_tiles, h->active_idx,
                     h->row_of_token, h->n_active, h->mask, h->quota_dev, h->dyn, h->dev_err, h->gemm_ws,
                     h->gemm_cnt, h->dec_scratch, h->dec_bits, h->dyn_curve, h->zero_quota, h->t_all,
                     h->freq_all, h->h1_all, h->temb_all, h->mod_all};
@@ -896,6 +898,7 @@ f3dc_status f3dc_create(const f3dc_config *cfg, const f3dc_weights *w, void *str
     CKC(dalloc(&h->plan, 1));
     CKC(cudaMemsetAsync(h->plan, 0, sizeof(Plan), s));
     CKC(dalloc(&h->tile_sample, (size_t)h->max_tiles));
+    CKC(dalloc(&h->pair_tiles, (size_t)h->max_tiles));
     CKC(dalloc(&h->active_idx, (size_t)B * N));
     CKC(dalloc(&h->row_of_token, (size_t)B * N));
     CKC(dalloc(&h->n_active, (size_t)B));
@@ -1098,6 +1101,7 @@ f3dc_status f3dc_step(f3dc_handle *h, int32_t k, int32_t B, float *S_inout, void
     a.row_of_token = h->row_of_token;
     a.plan = h->plan;
     a.tile_sample = h->tile_sample;
+    a.pair_tiles = h->pair_tiles;
     a.err = h->dev_err;
     h->last_B = B;
     Work w_sel;
@@ -1363,7 +1367,7 @@ f3dc_status f3dc_forward(f3dc_handle *h, float t, int32_t B, const float *S, con
     CK(cudaMemcpyAsync(h->active_idx, active_idx, (size_t)B * h->N * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     h->last_B = B;
     LAUNCH(KF_PLAN, Work(), launch_plan_from_counts(n_active, h->active_idx, B, h->N, h->plan, h->tile_sample,
-                                                    nullptr, h->dev_err, s));
+                                                    h->pair_tiles, nullptr, h->dev_err, s));
     f3dc_status st = run_dit(h, t, S, s);
     if (st != F3DC_OK) return st;
     LAUNCH(KF_SCATTER, wm(64.0), launch_scatter_rows(h->v_active, h->plan, B, h->N, v_out, s));

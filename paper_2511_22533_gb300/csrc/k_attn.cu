@@ -37,7 +37,7 @@
 // no branch on the data.
 // What bounds it: the softmax warps.  Per key tile of 128 x 128 scores an SM's
 // exponent unit needs 512 clocks (32 per clock) and the tensor core 512; the
-// kernel takes ~990 (4096 x 4096 x 16 heads, dh 64: 66.2 us = 1038 TFLOP/s;
+// kernel takes ~950 (4096 x 4096 x 16 heads, dh 64: 63.9 us = 1075 TFLOP/s;
 // before -- one issuer warp, a maximum of every half tile, ~1250 clocks --
 // 79.1 us; 1229 x 1374: 17.6 -> 15.9 us).  A softmax warp alone needs ~730
 // clocks per tile (load, exponents, store), and the two of an SM sub-partition
@@ -79,65 +79,42 @@ struct AttnCfg {
     static_assert(kColP + 128 <= kTmemCols, "TMEM layout");
 };
 
-// The key rows of query tile t: the sample's active tokens (self-attention),
-// the sample's condition tokens (cross-attention) or the one sequence.
-F3DC_DEV void tile_keys(const AttnParams &p, int t, int &kv_row0, int &nk)
-{
-    if (p.mode == 0) {
-        const int b = p.tile_sample[t];
-        kv_row0 = p.plan->row_off[b];
-        nk = p.plan->n_active[b];
-    } else if (p.mode == 1) {
-        const int b = p.tile_sample[t];
-        kv_row0 = (p.kv_null_from > 0 && b >= p.kv_null_from ? p.kv_null_sample : b) * p.nk_fixed;
-        nk = p.nk_fixed;
-    } else {
-        kv_row0 = 0;
-        nk = p.nk_fixed;
-    }
-}
-
 struct Item {
-    int q_row0, kv_row0, nk, h, store_end;  // q_row0: tile A's first row (B follows)
-    bool store[2];
+    int q_row0, kv_row0, nk, h;  // q_row0: tile A's first row (B follows)
+    bool both;                              // tile B is the pair's too (else computed, never stored)
 };
 
-// Work item w: query tiles A = 2 pt and B = 2 pt + 1 of head h, for the
-// first n_pt heads items (n_pt = tile pairs).  The two tiles share the keys,
-// so a pair whose tiles have different keys (two samples meet inside it)
-// runs twice: the first pass with tile A's keys stores only A's rows, a
-// second pass (items n_pt heads .. 2 n_pt heads - 1) with tile B's keys
-// stores only B's; any other second-pass item is skipped (returns false).
-// Rows of a tile beyond the tile count are computed and never stored.
-F3DC_DEV bool decode_item(const AttnParams &p, int w, int n_tiles, Item &it)
+// Work item w: pair w / heads of query tiles, head w % heads.  The tiles of a
+// pair share their keys: the plan lists pairs within one sample, at most one of
+// them half empty, and every listed sample has active tokens.  Pairs of
+// neighbours in the packed rows, run twice where two samples meet, did up to 20 %
+// more key tiles: a guided step of eight samples with 400 - 4096 active tokens
+// took 2636 us, with these pairs 2557 (self-attention 295 -> 270 us,
+// cross-attention 188 -> 170).  Items come longest first, one of every gridDim.x
+// for a CTA; walking them forwards and backwards in turn measured the same there
+// and 0.5 us slower at 4096 x 4096.
+F3DC_DEV void decode_item(const AttnParams &p, int w, int n_tiles, Item &it)
 {
-    it.store_end = p.mode == 2 ? p.q_rows : 0x7FFFFFFF;
-    const int per_pass = ((n_tiles + 1) >> 1) * p.heads;
-    const int pass = w >= per_pass ? 1 : 0;
-    const int w2 = w - pass * per_pass;
-    const int pt = w2 / p.heads;
-    it.h = w2 - pt * p.heads;
-    const int t0 = 2 * pt;
-    const bool has1 = t0 + 1 < n_tiles;
-    int r0, n0, r1, n1;
-    tile_keys(p, t0, r0, n0);
-    if (has1) {
-        tile_keys(p, t0 + 1, r1, n1);
-    } else {
-        r1 = r0;
-        n1 = n0;
+    const int pt = w / p.heads;
+    it.h = w - pt * p.heads;
+    if (p.mode == 2) {  // one sequence
+        it.q_row0 = 256 * pt;
+        it.both = 2 * pt + 1 < n_tiles;
+        it.kv_row0 = 0;
+        it.nk = p.nk_fixed;
+        return;
     }
-    const bool mixed = r1 != r0 || n1 != n0;
-    if (pass == 1 && !mixed) return false;
-    it.kv_row0 = pass ? r1 : r0;
-    it.nk = pass ? n1 : n0;
-    it.q_row0 = t0 * 128;
-    it.store[0] = pass == 0;
-    it.store[1] = has1 && (pass == 1 || !mixed);
-    return true;
+    const int e = p.pair_tiles[pt], b = (e & ~kPairBoth) >> kPairSampleShift;
+    it.q_row0 = (e & kPairTileMask) * 128;
+    it.both = (e & kPairBoth) != 0;
+    if (p.mode == 0) {  // the sample's active tokens
+        it.kv_row0 = p.plan->row_off[b];
+        it.nk = p.plan->n_active[b];
+    } else {  // the sample's condition tokens
+        it.kv_row0 = (p.kv_null_from > 0 && b >= p.kv_null_from ? p.kv_null_sample : b) * p.nk_fixed;
+        it.nk = p.nk_fixed;
+    }
 }
-
-F3DC_DEV int total_items(const AttnParams &p, int n_tiles) { return 2 * ((n_tiles + 1) >> 1) * p.heads; }
 
 F3DC_DEV bool wait_bounded(uint64_t *bar, uint32_t parity, uint64_t ns)
 {
@@ -216,7 +193,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // the previous kernel's outputs (Q / K / V, the row plan) are complete
     griddep_wait();
     const int n_tiles = __shfl_sync(0xffffffffu, p.n_tiles_dev ? *p.n_tiles_dev : p.n_tiles, 0);
-    const int total = total_items(p, n_tiles);
+    const int total =
+        (p.n_tiles_dev ? __shfl_sync(0xffffffffu, p.plan->n_pairs, 0) : (n_tiles + 1) >> 1) * p.heads;
 
     // Every warp ends a pass over the CTA's items here, also when the kernel is
     // aborting (each role's waits are bounded); a second pass follows if the
@@ -242,7 +220,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll 1
                 for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
                     Item it;
-                    if (!decode_item(p, w, n_tiles, it)) continue;
+                    decode_item(p, w, n_tiles, it);
                     const uint32_t my_it = item_it++;
                     // Q buffer qb holds items qb, qb + 2, ...: its (my_it / 2)-th use
                     const uint32_t qb = my_it & 1, qph = (my_it >> 1) & 1;
@@ -311,11 +289,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     if (j == nkt) {  // the next real work item
                         if (nkt) ++item;
                         nkt = j = 0;
-#pragma unroll 1
-                        while (nkt == 0 && (w += gridDim.x) < total) {
+                        if ((w += gridDim.x) < total) {
                             Item it;
-                            const uint32_t n = decode_item(p, w, n_tiles, it) ? (uint32_t)((it.nk + 127) / 128) : 0u;
-                            nkt = __shfl_sync(0xffffffffu, n, 0);
+                            decode_item(p, w, n_tiles, it);
+                            nkt = __shfl_sync(0xffffffffu, (uint32_t)((it.nk + 127) / 128), 0);
                         }
                     }
                     if (nkt) {
@@ -487,18 +464,26 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll 1
             for (int w = blockIdx.x; w < total; w += gridDim.x) {
                 Item it;
-                const int nk = __shfl_sync(0xffffffffu, decode_item(p, w, n_tiles, it) ? it.nk : 0, 0);
-                if (nk == 0) continue;
+                decode_item(p, w, n_tiles, it);
+                const int nk = __shfl_sync(0xffffffffu, it.nk, 0);
                 m_ref = -INFINITY;
                 l_run = 0.f;
                 bool ok = true;
+                // The plain tiles run in a loop of their own, with as few values
+                // kept over it as can be: one loop that picks each tile's form,
+                // and one more value in it, cost register moves (4096 x 4096:
+                // 66.5 us, here 63.9).
+                int left = nk;
+                bool first = true;
+                do {
+                    ok = max_tile(g++, first, left);
+                    left -= 128;
+                    first = false;
+                    if (pass == 0) {
 #pragma unroll 1
-                for (int k0 = 0; k0 < nk && ok; k0 += 128, ++g) {
-                    if (k0 > 0 && nk - k0 >= 128 && pass == 0)
-                        ok = plain_tile(g);
-                    else
-                        ok = max_tile(g, k0 == 0, nk - k0);
-                }
+                        for (; ok && left >= 128; left -= 128) ok = plain_tile(g++);
+                    }
+                } while (ok && left > 0);
                 if (!ok) break;
                 // every P V of the item done: O_t / l, stored as bf16
                 if (!wait(&pv_done[t], (g - 1) & 1)) break;
@@ -516,7 +501,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&o_free[t]);
                 const int orow = it.q_row0 + 128 * t + row;
-                if (it.store[t] && orow < it.store_end) {
+                if ((t == 0 || it.both) && orow < p.q_rows) {
                     // The first pass takes the reference from the item's first
                     // key tile.  P, l and O carry it exactly as long as no
                     // exponent overflows (all three have 8 exponent bits), and

@@ -108,6 +108,9 @@ F3DC_DEV uint32_t score_key(float s)
 
 F3DC_DEV int pad_tile(int a) { return (a + kTileRows - 1) / kTileRows * kTileRows; }
 
+// pairs of tiles that n active tokens fill
+F3DC_DEV int tile_pairs(int n) { return (n + 2 * kTileRows - 1) / (2 * kTileRows); }
+
 F3DC_DEV int clamp_quota(int q, int N) { return q < 0 ? 0 : (q > N ? N : q); }
 
 // Distributed shared memory: the address of a variable in CTA `rank` of the
@@ -123,26 +126,34 @@ F3DC_DEV float ld_dsmem_f32(uint32_t addr) { return __uint_as_float(ld_dsmem_u32
 F3DC_DEV void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 F3DC_DEV void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// Row offset of sample b, total padded rows, and the sample's tiles.  The
-// first warp sums the padded row counts of all samples (B <= 64: two per
-// lane) in one round of loads.  Every CTA of the cluster computes the
+// Row offset of sample b, total padded rows, and the sample's tiles and pairs
+// of tiles.  The first warp sums the padded row counts of all samples (B <= 64:
+// two per lane) in one round of loads, and the pairs of those that come before
+// (more active tokens, then the lower number; a guided step's copy follows its
+// sample).  Every CTA of the cluster computes the
 // offset; only the cluster's first CTA (`writer`) writes the plan.
 static_assert(kMaxBatch <= 64, "write_plan covers two samples per lane");
 F3DC_DEV void write_plan(const SelectArgs &a, int b, int na, bool writer, int &off)
 {
-    __shared__ int s_off, s_tot_rows;
+    __shared__ int s_off, s_tot_rows, s_pair0;
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        const int r0 = lane < a.B ? pad_tile(a.N - clamp_quota(a.quota[lane], a.N)) : 0;
-        const int r1 = lane + 32 < a.B ? pad_tile(a.N - clamp_quota(a.quota[lane + 32], a.N)) : 0;
+        const int n0 = lane < a.B ? a.N - clamp_quota(a.quota[lane], a.N) : 0;
+        const int n1 = lane + 32 < a.B ? a.N - clamp_quota(a.quota[lane + 32], a.N) : 0;
+        const int r0 = pad_tile(n0), r1 = pad_tile(n1), p0 = tile_pairs(n0), p1 = tile_pairs(n1);
         int before = (lane < b ? r0 : 0) + (lane + 32 < b ? r1 : 0), tot = r0 + r1;
+        int pair0 = (n0 > na || (n0 == na && lane < b) ? p0 : 0) + (n1 > na || (n1 == na && lane + 32 < b) ? p1 : 0);
+        int pairs = p0 + p1;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             before += __shfl_xor_sync(0xffffffffu, before, o);
             tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            pair0 += __shfl_xor_sync(0xffffffffu, pair0, o);
+            pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
         }
         if (lane == 0) {
             s_off = before;
+            s_pair0 = pair0;
             s_tot_rows = tot;
             if (a.plan && writer) {
                 a.plan->n_active[b] = na;
@@ -155,6 +166,7 @@ F3DC_DEV void write_plan(const SelectArgs &a, int b, int na, bool writer, int &o
                     const int all = a.cfg_dup ? 2 * tot : tot;
                     a.plan->m_rows = all;
                     a.plan->n_tiles = all / kTileRows;
+                    a.plan->n_pairs = a.cfg_dup ? 2 * pairs : pairs;
                 }
             }
         }
@@ -167,6 +179,12 @@ F3DC_DEV void write_plan(const SelectArgs &a, int b, int na, bool writer, int &o
         if (a.cfg_dup) {
             const int t1 = (s_tot_rows + off) / kTileRows;
             for (int t = threadIdx.x; t < nt; t += blockDim.x) a.tile_sample[t1 + t] = a.B + b;
+        }
+        const int np = (nt + 1) / 2, copies = a.cfg_dup ? 2 : 1;
+        for (int i = threadIdx.x; i < copies * np; i += blockDim.x) {
+            const int copy = i >= np, j = 2 * (i - copy * np);
+            a.pair_tiles[copies * s_pair0 + i] =
+                tile_pair(t0 + copy * (s_tot_rows / kTileRows) + j, b + copy * a.B, j + 1 < nt);
         }
     }
 }
@@ -495,13 +513,13 @@ __global__ void __cluster_dims__(kSelCS, 1, 1) __launch_bounds__(kSelThreads, 4)
 }
 
 __global__ void k_plan_from_counts(const int32_t *n_active, int B, int N, Plan *plan, int32_t *tile_sample,
-                                   uint32_t *err)
+                                   int32_t *pair_tiles, uint32_t *err)
 {
     griddep_launch();
     griddep_wait();
-    __shared__ int offs[kMaxBatch + 1];
+    __shared__ int offs[kMaxBatch + 1], s_na[kMaxBatch], pair0[kMaxBatch];
     if (threadIdx.x == 0) {
-        int o = 0;
+        int o = 0, pairs = 0;
         for (int b = 0; b < B; ++b) {
             int na = n_active[b];
             if (na < 0 || na > N) {
@@ -511,16 +529,29 @@ __global__ void k_plan_from_counts(const int32_t *n_active, int B, int N, Plan *
             offs[b] = o;
             plan->n_active[b] = na;
             plan->row_off[b] = o;
+            s_na[b] = na;
             o += pad_tile(na);
+            pairs += tile_pairs(na);
         }
         offs[B] = o;
         plan->m_rows = o;
         plan->n_tiles = o / kTileRows;
+        plan->n_pairs = pairs;
+    }
+    __syncthreads();
+    if (threadIdx.x < B) {
+        const int b = threadIdx.x;
+        int p = 0;
+        for (int o = 0; o < B; ++o)
+            if (s_na[o] > s_na[b] || (s_na[o] == s_na[b] && o < b)) p += tile_pairs(s_na[o]);
+        pair0[b] = p;
     }
     __syncthreads();
     for (int b = 0; b < B; ++b) {
         const int t0 = offs[b] / kTileRows, t1 = offs[b + 1] / kTileRows;
         for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) tile_sample[t] = b;
+        for (int t = t0 + 2 * threadIdx.x; t < t1; t += 2 * blockDim.x)
+            pair_tiles[pair0[b] + (t - t0) / 2] = tile_pair(t, b, t + 1 < t1);
     }
 }
 
@@ -558,13 +589,14 @@ cudaError_t launch_ssc_select(const SelectArgs &a, cudaStream_t s)
 }
 
 cudaError_t launch_plan_from_counts(const int32_t *n_active, const int32_t *active_idx, int B, int N,
-                                    Plan *plan, int32_t *tile_sample, int32_t *row_of_token, uint32_t *err,
-                                    cudaStream_t s)
+                                    Plan *plan, int32_t *tile_sample, int32_t *pair_tiles, int32_t *row_of_token,
+                                    uint32_t *err, cudaStream_t s)
 {
     (void)active_idx;
     (void)row_of_token;
     if (B < 1 || B > kMaxBatch) return cudaErrorInvalidValue;
-    launch_k(k_plan_from_counts, dim3(1), dim3(256), 0, s, n_active, B, N, plan, tile_sample, err);
+    launch_k(k_plan_from_counts, dim3(1), dim3(256), 0, s, n_active, B, N, plan, tile_sample, pair_tiles,
+             err);
     return cudaGetLastError();
 }
 

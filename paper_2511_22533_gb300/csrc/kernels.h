@@ -20,13 +20,25 @@ typedef __nv_bfloat16 bf16;
 // Per-step row plan.  Active tokens of all samples are packed row-wise,
 // sample b's a_b rows starting at row_off[b] (a multiple of 128) and padded
 // to a multiple of 128 with finite rows, so every 128-row tile belongs to
-// one sample (tile_sample[] in a separate array).
+// one sample (tile_sample[] in a separate array).  For attention the tiles are
+// listed as pairs of one sample (pair_tiles[], see tile_pair), the samples with
+// most active tokens first.
 struct Plan {
     int32_t n_tiles;               // padded rows / 128
+    int32_t n_pairs;               // entries of pair_tiles
     int32_t m_rows;                // padded rows
     int32_t n_active[kMaxBatch];   // a_b
     int32_t row_off[kMaxBatch];    // first packed row of sample b
 };
+
+// Entry of pair_tiles: first tile, sample, and whether the next tile belongs to
+// the pair (the last pair of a sample with an odd number of tiles has one).
+constexpr int32_t kPairTileMask = 0xFFFFF, kPairSampleShift = 20, kPairBoth = 1 << 30;
+static_assert(kMaxBatch <= 1 << 10, "a sample's number fits its field");
+__host__ __device__ inline int32_t tile_pair(int tile, int sample, bool both)
+{
+    return tile | sample << kPairSampleShift | (both ? kPairBoth : 0);
+}
 
 // ------------------------------------------------------------ selection
 struct SelectArgs {
@@ -41,6 +53,7 @@ struct SelectArgs {
     int32_t *row_of_token;     // [B, N], nullable: packed row or -1 if cached
     Plan *plan;                // nullable
     int32_t *tile_sample;      // nullable
+    int32_t *pair_tiles;       // written with tile_sample
     // guided (CFG) step: the plan also lists samples B..2B-1, copies of
     // samples 0..B-1 (same active counts, rows after all of 0..B-1's)
     int cfg_dup;
@@ -50,10 +63,10 @@ cudaError_t launch_ssc_select(const SelectArgs &a, cudaStream_t s);
 int ssc_select_max_tokens();
 
 // Plan from given active lists (diagnostic forward): counts -> plan,
-// tile_sample and row_of_token.
+// tile_sample, pair_tiles and row_of_token.
 cudaError_t launch_plan_from_counts(const int32_t *n_active, const int32_t *active_idx, int B, int N,
-                                    Plan *plan, int32_t *tile_sample, int32_t *row_of_token, uint32_t *err,
-                                    cudaStream_t s);
+                                    Plan *plan, int32_t *tile_sample, int32_t *pair_tiles, int32_t *row_of_token,
+                                    uint32_t *err, cudaStream_t s);
 
 // ------------------------------------------------------------ row kernels
 // x[r] = in_w S[b, i] + in_b + pos[i] for packed active row r; zero pad rows.
@@ -248,10 +261,11 @@ struct AttnParams {
     int mode;                      // 0 self (plan), 1 cross (b * nk_fixed), 2 single sequence
     const int32_t *n_tiles_dev;    // nullable
     int n_tiles;
-    const int32_t *tile_sample;    // modes 0, 1
-    const Plan *plan;              // mode 0
+    const int32_t *tile_sample;    // modes 0, 1 (one-tile kernel)
+    const int32_t *pair_tiles;     // modes 0, 1 (pair kernel)
+    const Plan *plan;              // modes 0, 1
     int nk_fixed;                  // modes 1, 2
-    int q_rows;                    // mode 2: rows stored are < q_rows
+    int q_rows;                    // rows stored are < q_rows
     bf16 *out;
     int ldo;
     float scale_log2;              // log2(e) / sqrt(dh)

@@ -163,3 +163,36 @@ def test_cfg_trellis_width_step(orc):
     amax, l2 = _guided_bound(vc, vu, s)
     assert np.all(np.abs(got - ref) <= amax + bf16_ulp(np.maximum(np.abs(got), np.abs(ref)))), max_abs(got, ref)
     h.close()
+
+
+def test_cfg_step_of_pairs_at_the_edges(orc):
+    # the attention takes query tiles in pairs of one sample, most active tokens
+    # first: samples of 1, 129 (two tiles), 0, 512 and 257 (three tiles, so half
+    # of the last pair is empty) tokens, each with its unguided copy
+    s, active = 2.0, [1, 129, 0, 512, 257]
+    B = len(active)
+    h, blob, _ = handle_for(TINY, max_batch=B, cfg_strength=s, cfg_t_lo=0.0)
+    m = orc.Model(TINY, blob)
+    cond = synth.cond_tokens(TINY, B, 0)
+    S = synth.latents(TINY, B, 0)
+    h.set_cond(dev_u16(cond), B)
+    kv_u = m.cond_kv(np.zeros_like(cond[0]))
+    hist = synth.velocity_history(8, 8, B, seed=9)
+    quotas = 512 - np.array(active, np.int32)
+    k = 4
+    vt_gpu, S_gpu = _step(h, S, k, quotas, hist)
+    for b in range(B):
+        cached, idx, vc, vu, S_o, vt_o = _oracle_step(orc, m, S[b], k, quotas[b], hist[:, b], m.cond_kv(cond[b]),
+                                                       kv_u, s, TINY.steps)
+        assert len(idx) == active[b]
+        cm = cached.astype(bool)
+        np.testing.assert_array_equal(vt_gpu[b][cm], hist[2, b][cm])
+        np.testing.assert_array_equal(S_gpu[b][cm], S_o[cm])
+        if not len(idx):
+            continue
+        got = synth.bf16_bits_to_f32(vt_gpu[b][idx])
+        ref = synth.bf16_bits_to_f32(vt_o[idx])
+        amax, l2 = _guided_bound(vc, vu, s)
+        assert np.all(np.abs(got - ref) <= amax + bf16_ulp(np.maximum(np.abs(got), np.abs(ref)))), (b, max_abs(got, ref))
+        assert np.linalg.norm(got.astype(np.float64) - ref) <= l2 + np.sqrt(got.size) * 2.0 ** -8 * np.abs(ref).max()
+    h.close()

@@ -85,6 +85,20 @@ def test_forward_tiny_ragged_subsets(tiny):
         _assert_vel(got[b], tiny.m.forward(tiny.S[b], lists[b], 0.6, tiny.kv[b]), f"sample {b}")
 
 
+def test_forward_pairs_of_tiles_at_the_edges(orc):
+    # as many tokens as fill an odd and an even number of tiles, none, equal counts
+    counts = [129, 0, 512, 257, 129, 1]
+    c = Ctx(orc, TINY, len(counts))
+    g = np.random.default_rng(5)
+    lists = [np.sort(g.choice(512, n, replace=False)) for n in counts]
+    got = _forward_gpu(c.h, 0.5, c.S, lists)
+    for b, n in enumerate(counts):
+        if n:
+            _assert_vel(got[b], c.m.forward(c.S[b], lists[b], 0.5, c.kv[b]), f"sample {b}")
+    assert_clean(c.h)
+    c.h.close()
+
+
 def test_forward_single_token_and_empty(tiny):
     lists = [np.array([511]), np.array([], np.int64)]
     got = _forward_gpu(tiny.h, 0.3, tiny.S, lists)
