@@ -93,8 +93,11 @@ struct Item {
 // cross-attention 188 -> 170).  Items come longest first, one of every gridDim.x
 // for a CTA; walking them forwards and backwards in turn measured the same there
 // and 0.5 us slower at 4096 x 4096.
+// kEarly: before griddep_wait (the plan is read from L2).
+template <bool kEarly = false>
 F3DC_DEV void decode_item(const AttnParams &p, int w, int n_tiles, Item &it)
 {
+    auto ld = [](const int32_t *q) { return kEarly ? ld_plan(q) : *q; };
     const int pt = w / p.heads;
     it.h = w - pt * p.heads;
     if (p.mode == 2) {  // one sequence
@@ -104,12 +107,12 @@ F3DC_DEV void decode_item(const AttnParams &p, int w, int n_tiles, Item &it)
         it.nk = p.nk_fixed;
         return;
     }
-    const int e = p.pair_tiles[pt], b = (e & ~kPairBoth) >> kPairSampleShift;
+    const int e = ld(p.pair_tiles + pt), b = (e & ~kPairBoth) >> kPairSampleShift;
     it.q_row0 = (e & kPairTileMask) * 128;
     it.both = (e & kPairBoth) != 0;
     if (p.mode == 0) {  // the sample's active tokens
-        it.kv_row0 = p.plan->row_off[b];
-        it.nk = p.plan->n_active[b];
+        it.kv_row0 = ld(p.plan->row_off + b);
+        it.nk = ld(p.plan->n_active + b);
     } else {  // the sample's condition tokens
         it.kv_row0 = (p.kv_null_from > 0 && b >= p.kv_null_from ? p.kv_null_sample : b) * p.nk_fixed;
         it.nk = p.nk_fixed;
@@ -177,6 +180,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         tmem_alloc(tmem_holder, Cfg::kTmemCols);
         tmem_relinquish();
     }
+    if (warp == 0 && lane == 0) {
+        tma_prefetch(&tmq);
+        tma_prefetch(&tmk);
+        tma_prefetch(&tmv);
+    }
     if (p.kv_prefetch_rows > 0 && warp == 0 && lane == 0) {
         // keys / values written long before this launch (the condition's):
         // pull this CTA's share into L2 while the previous kernel finishes
@@ -190,11 +198,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
-    // the previous kernel's outputs (Q / K / V, the row plan) are complete
-    griddep_wait();
-    const int n_tiles = __shfl_sync(0xffffffffu, p.n_tiles_dev ? *p.n_tiles_dev : p.n_tiles, 0);
+    const int n_tiles = __shfl_sync(0xffffffffu, p.n_tiles_dev ? ld_plan(p.n_tiles_dev) : p.n_tiles, 0);
     const int total =
-        (p.n_tiles_dev ? __shfl_sync(0xffffffffu, p.plan->n_pairs, 0) : (n_tiles + 1) >> 1) * p.heads;
+        (p.n_tiles_dev ? __shfl_sync(0xffffffffu, ld_plan(&p.plan->n_pairs), 0) : (n_tiles + 1) >> 1) * p.heads;
+    // the producer's first item is looked up early: its loads are the first
+    // thing after the wait
+    Item first_item;
+    if (warp == 0 && (int)blockIdx.x < total) decode_item<true>(p, blockIdx.x, n_tiles, first_item);
+    // the previous kernel's outputs (Q / K / V) are complete
+    griddep_wait();
 
     // Every warp ends a pass over the CTA's items here, also when the kernel is
     // aborting (each role's waits are bounded); a second pass follows if the
@@ -211,16 +223,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             if (lane == 0) {
-                if (pass == 0) {
-                    tma_prefetch(&tmq);
-                    tma_prefetch(&tmk);
-                    tma_prefetch(&tmv);
-                }
                 bool ok = true;
 #pragma unroll 1
                 for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
-                    Item it;
-                    decode_item(p, w, n_tiles, it);
+                    Item it = first_item;
+                    if (w != (int)blockIdx.x) decode_item(p, w, n_tiles, it);
                     const uint32_t my_it = item_it++;
                     // Q buffer qb holds items qb, qb + 2, ...: its (my_it / 2)-th use
                     const uint32_t qb = my_it & 1, qph = (my_it >> 1) & 1;

@@ -76,19 +76,22 @@ struct Item {
     int q_row0, kv_row0, nk, h, store_end;
 };
 
+// kEarly: before griddep_wait (the plan is read from L2).
+template <bool kEarly = false>
 F3DC_DEV Item decode_item(const AttnParams &p, int w)
 {
+    auto ld = [](const int32_t *q) { return kEarly ? ld_plan(q) : *q; };
     Item it;
     const int t = w / p.heads;
     it.h = w - t * p.heads;
     it.q_row0 = t * 128;
     it.store_end = 0x7FFFFFFF;
     if (p.mode == 0) {
-        const int b = p.tile_sample[t];
-        it.kv_row0 = p.plan->row_off[b];
-        it.nk = p.plan->n_active[b];
+        const int b = ld(p.tile_sample + t);
+        it.kv_row0 = ld(p.plan->row_off + b);
+        it.nk = ld(p.plan->n_active + b);
     } else if (p.mode == 1) {
-        const int b = p.tile_sample[t];
+        const int b = ld(p.tile_sample + t);
         it.kv_row0 = (p.kv_null_from > 0 && b >= p.kv_null_from ? p.kv_null_sample : b) * p.nk_fixed;
         it.nk = p.nk_fixed;
     } else {
@@ -199,6 +202,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         tmem_alloc(tmem_holder, Cfg::kTmemCols);
         tmem_relinquish();
     }
+    if (warp == 0 && lane == 0) {
+        tma_prefetch(&tmq);
+        tma_prefetch(&tmk);
+        tma_prefetch(&tmv);
+    }
     if (p.kv_prefetch_rows > 0 && warp == 0 && lane == 0) {
         // keys / values written long before this launch (the condition's):
         // pull this CTA's share into L2 while the previous kernel finishes
@@ -212,21 +220,22 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
-    // the previous kernel's outputs (Q / K / V, the row plan) are complete
-    griddep_wait();
-    const int n_tiles = p.n_tiles_dev ? *p.n_tiles_dev : p.n_tiles;
+    const int n_tiles = p.n_tiles_dev ? ld_plan(p.n_tiles_dev) : p.n_tiles;
     const int total = n_tiles * p.heads;
+    // the producer's first item is looked up early: its loads are the first
+    // thing after the wait
+    Item first_item;
+    if (warp == 0 && (int)blockIdx.x < total) first_item = decode_item<true>(p, blockIdx.x);
+    // the previous kernel's outputs (Q / K / V) are complete
+    griddep_wait();
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         if (lane == 0) {
-            tma_prefetch(&tmq);
-            tma_prefetch(&tmk);
-            tma_prefetch(&tmv);
             uint32_t kv_it = 0, item_it = 0;
             bool ok = true;
             for (int w = blockIdx.x; w < total && ok; w += gridDim.x, ++item_it) {
-                const Item it = decode_item(p, w);
+                const Item it = w == (int)blockIdx.x ? first_item : decode_item(p, w);
                 // buffer qb holds items qb, qb + 2, ...: its (item_it / 2)-th use
                 const uint32_t qb = item_it & 1, qph = (item_it >> 1) & 1;
                 if (!mbar_wait(&q_empty[qb], qph ^ 1, abort_flag, p.err)) break;

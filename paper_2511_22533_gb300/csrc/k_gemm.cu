@@ -403,10 +403,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_holder;
-    // the previous kernel's outputs (A, the row plan, x) are complete
-    griddep_wait();
     Units U;
-    U.m_tiles = p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles;
+    U.m_tiles = p.m_tiles_dev ? ld_plan(p.m_tiles_dev) : p.m_tiles;
+    // the previous kernel's outputs (A, x) are complete
+    griddep_wait();
     U.tiles = U.m_tiles * (p.N / BN);
     U.kb_n = p.K / kBK;
     U.splits = gemm_split_count(U.tiles, (int)gridDim.x, U.kb_n, p.ws_units, p.ws != nullptr);
@@ -733,11 +733,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         for (int i = blockIdx.x; i < boxes; i += gridDim.x)
             tma_prefetch_l2_3d(&tmb.rows[0], 0, (i / kbx) * 128, (i % kbx) * 2);
     }
-    griddep_wait();
-    const int m_tiles = __shfl_sync(0xffffffffu, p.m_tiles_dev ? *p.m_tiles_dev : p.m_tiles, 0);
+    const int m_tiles = __shfl_sync(0xffffffffu, p.m_tiles_dev ? ld_plan(p.m_tiles_dev) : p.m_tiles, 0);
     const int kb_n = p.K / kPairBK;
     const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
     const PairUnits U((m_tiles + 1) / 2, p.N, ncl, p.M);
+    griddep_wait();  // the previous kernel's outputs (A, x) are complete
     // The tensor core truncates as it accumulates, so the error of a sum grows
     // with its length (4096: 3.2e-6 relative, 1024: 7e-7).  A long K is summed
     // in pieces where the second TMEM buffer is not needed for a next unit:

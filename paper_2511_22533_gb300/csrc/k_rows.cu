@@ -69,8 +69,10 @@ __global__ void __launch_bounds__(GatherCfg<NV>::kThreads, GatherCfg<NV>::kThrea
         bf16x8_to_f32(__ldg(reinterpret_cast<const uint4 *>(in_w) + 4 * q + u), wv[u]);
         bv[u] = bf16_at(in_b, 4 * q + u);
     }
-    griddep_launch();
+    // in this order: the kernels after this one read the row plan and the
+    // modulation before their own wait (see griddep_wait)
     griddep_wait();
+    griddep_launch();
     const int units = plan->m_rows / kGatherUnit;
     for (int unit = blockIdx.x; unit < units; unit += gridDim.x) {
         const int r0 = unit * kGatherUnit;
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(GatherCfg<NV>::kThreads, GatherCfg<NV>::kThrea
 // ------------------------------------------------------------------ K7
 // One warp per row, lane l owning float4 columns q * 32 + l.  The per-column
 // modulation (adaLN scale / shift, or LN gain / bias) is staged in shared
-// memory once per CTA while the first row is in flight, and each warp loads
+// memory once per CTA while the previous kernel finishes, and each warp loads
 // its next row while it normalises the current one, so the kernel streams
 // rows at a persistent grid of two CTAs per SM instead of paying two
 // dependent memory round trips per row.
@@ -139,26 +141,22 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_layernorm(const float *x, in
                                                               const bf16 *g, const bf16 *bb, bf16 *out)
 {
     griddep_launch();
-    griddep_wait();
     __shared__ float4 s_mul[NV * 32], s_add[NV * 32];  // y = xhat * mul + add per column
-    const int m_rows = plan->m_rows;
+    const int m_rows = ld_plan(&plan->m_rows);
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int stride = gridDim.x * wpb;
     int r = blockIdx.x * wpb + (threadIdx.x >> 5);
-    if (blockIdx.x * wpb >= m_rows) return;  // the whole CTA is idle
-    // the first row's loads are issued before the modulation is staged, so
-    // the two memory round trips overlap
-    float4 v[NV];
-    if (r < m_rows) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) v[q] = ld_f4(x + (size_t)r * W + 4 * (q * 32 + lane));
+    if (blockIdx.x * wpb >= m_rows) {  // the whole CTA is idle
+        griddep_wait();
+        return;
     }
+    // the modulation is staged while the previous kernel finishes
     for (int c4 = threadIdx.x; c4 < NV * 32; c4 += blockDim.x) {
         const int n0 = 4 * c4;
         if (mode == 0) {
-            const float4 sc = ld_f4(scale + n0);
+            const float4 sc = __ldcg(reinterpret_cast<const float4 *>(scale + n0));
             s_mul[c4] = make_float4(1.f + sc.x, 1.f + sc.y, 1.f + sc.z, 1.f + sc.w);
-            s_add[c4] = ld_f4(shift + n0);
+            s_add[c4] = __ldcg(reinterpret_cast<const float4 *>(shift + n0));
         } else {
             const uint2 gw = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(g) + n0));
             const uint2 bw = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(bb) + n0));
@@ -167,6 +165,12 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_layernorm(const float *x, in
             s_add[c4] = make_float4(bf16_bits_to_f32(bw.x & 0xFFFFu), bf16_bits_to_f32(bw.x >> 16),
                                     bf16_bits_to_f32(bw.y & 0xFFFFu), bf16_bits_to_f32(bw.y >> 16));
         }
+    }
+    griddep_wait();
+    float4 v[NV];
+    if (r < m_rows) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) v[q] = ld_f4(x + (size_t)r * W + 4 * (q * 32 + lane));
     }
     __syncthreads();
     if (r >= m_rows) return;
@@ -198,8 +202,8 @@ __global__ void __launch_bounds__(kRowThreads) k_final_layer(const float *x, int
                                                              const bf16 *out_w, const bf16 *out_b, float *v_active)
 {
     griddep_launch();
+    const int m_rows = ld_plan(&plan->m_rows);
     griddep_wait();
-    const int m_rows = plan->m_rows;
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < m_rows; r += gridDim.x * wpb) {
         const float *xr = x + (size_t)r * W;

@@ -13,9 +13,9 @@
 // order-preserving 32-bit key per token (in place of V), and a 4 x 8-bit
 // radix select finds the c-th smallest key of the sample: every CTA counts
 // its keys into a 256-bin histogram, the cluster sums the eight histograms
-// bin by bin (each CTA redundantly, so all take the same digit), and ends at the first digit whose keys are all
-// cached.  Finally
-// each CTA caches its keys below the threshold plus the lowest-index ties
+// bin by bin (each CTA redundantly, so all take the same digit), and the
+// search ends at the first digit whose keys are all cached.  Finally each CTA
+// caches its keys below the threshold plus the lowest-index ties
 // and compacts its active tokens in ascending order, starting from the
 // counts of the lower-ranked CTAs.  With a third history slot (SSC with
 // three predictions) the acceleration term is the second difference of the
