@@ -509,7 +509,11 @@ cudaError_t run_attention(f3dc_handle *h, int mode, const CUtensorMap &tq, const
     p.err = h->dev_err;
     // persistent CTAs, one per work item up to one per SM: (query tile, head)
     // items for the one-tile kernel, (pair of query tiles, head) otherwise
-    const bool one = h->attn_one_now;
+    // One key tile (at most 128 condition tokens) gives the one-tile kernel
+    // nothing to share between its two chains, and pairs halve the items: a
+    // sample of the 8^3 model (256 x 64 keys x 4 heads) takes 948 us with pairs
+    // there, 970 without (alone, the launch takes 5.0 us against 4.6).
+    const bool one = h->attn_one_now && (mode == 0 || h->Nc > 128);
     const int per_sample = (h->N + kTileRows - 1) / kTileRows;  // tiles; pairs are within a sample
     const int items = (one ? h->max_tiles : h->max_tiles / per_sample * ((per_sample + 1) / 2)) * h->H;
     const int grid = items < h->num_sms ? items : h->num_sms;
