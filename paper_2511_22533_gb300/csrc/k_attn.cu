@@ -30,8 +30,9 @@
 // The reference m is the row's maximum over the item's first key tile (and
 // the ragged last one, if it is 2^8 above).  A later score above m is no
 // loss: P, l and O are floating point, with the same 8 exponent bits, so only
-// an overflow would be, and that is seen at the item's end (l above 2^64, O
-// not finite).  The CTA then does its items a second time with the maximum of
+// an overflow would be, and a ragged tile's raise whose factor underflows.  Both
+// are seen at the item's end (l above 2^64, O not finite; such a raise makes l
+// infinite).  The CTA then does its items a second time with the maximum of
 // every key tile, m raised (O_t and l rescaled in place) when a tile's maximum
 // is 2^8 above it.  So the loop over the key tiles takes no maximum and has
 // no branch on the data.
@@ -420,7 +421,12 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         // A key tile with its maximum (of its `valid` first keys): the item's
         // first and a ragged last one, and every one of a second pass.  The
         // reference is raised (O_t and l rescaled) when it grew by more than 2^8.
-        auto max_tile = [&](uint32_t g, bool first, int valid) {
+        // In a first pass the plain tiles before a ragged last one may lie far
+        // above the reference, up to this tile's maximum: a raise above 2^126,
+        // whose factor ex2.approx.ftz flushes to 0, would erase what they
+        // summed, so l becomes infinite instead and the item's end asks for the
+        // second pass.  (There an erased key is below 2^-118 of the row.)
+        auto max_tile = [&](uint32_t g, bool first, int valid, bool second_pass) {
             float sv[128];
             if (!load_s(g, sv)) return false;
             if (valid < 128) {
@@ -440,8 +446,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             if (__any_sync(0xffffffffu, mx > m_ref + 8.0f)) {
                 const float m_new = fmaxf(m_ref, mx);
                 const float alpha = exp2_fast(m_ref - m_new);
+                if (!first && !second_pass && m_new - m_ref > 126.0f) l_run = INFINITY;
+                else l_run *= alpha;
                 m_ref = m_new;
-                l_run *= alpha;
                 if (!first) {  // O_t holds this item's earlier tiles
 #pragma unroll 1
                     for (int d0 = 0; d0 < DH; d0 += 16) {
@@ -483,7 +490,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 int left = nk;
                 bool first = true;
                 do {
-                    ok = max_tile(g++, first, left);
+                    ok = max_tile(g++, first, left, pass != 0);
                     left -= 128;
                     first = false;
                     if (pass == 0) {

@@ -159,3 +159,32 @@ def test_attention_first_pass_reference_is_not_enough(orc, nq, nk, H, dh, kind):
     assert np.isfinite(got).all()
     assert rel_l2(got / scale, ref / scale) < 1e-2
     assert np.max(np.abs(got - ref)) / scale < 2e-2
+
+
+@pytest.mark.parametrize("nq,nk,H,dh", [(1280, 257, 16, 64), (2600, 257, 8, 32), (1280, 385, 16, 64)])
+@pytest.mark.parametrize("middle,last", [(119.0, 127.0), (117.0, 125.0), (133.0, 140.0), (60.0, 187.0)])
+def test_attention_ragged_last_tile_far_above_the_first(orc, nq, nk, H, dh, middle, last):
+    # scaled scores (log2 units) of 0 in the first key tile, `middle` in the
+    # plain tiles after it and `last` on the one key of the ragged last tile:
+    # raising the reference by more than 2^126 there flushes the factor that
+    # rescales l and O to 0, while the plain tiles, 2^8 below the last key and
+    # 128 keys strong, hold a third of the row's weight
+    g = np.random.default_rng(nq + nk)
+    W = H * dh
+    u = np.where(g.random((H, dh)) < 0.5, -1.0, 1.0)
+    q = np.broadcast_to(u.reshape(1, W), (nq, W))
+    unit = 1.0 / (np.sqrt(dh) * np.log2(np.e))
+    a = np.zeros(nk)
+    a[128:nk - 1] = middle * unit
+    a[nk - 1] = last * unit
+    k = np.einsum("j,hd->jhd", a, u).reshape(nk, W)
+    v = np.where(np.arange(nk)[:, None] == nk - 1, -0.5, 0.5) + 0.05 * g.standard_normal((nk, W))
+    qb, kb, vb = (synth.f32_to_bf16_bits(x.astype(np.float32)) for x in (q, k, v))
+    out = torch.zeros((nq, W), dtype=torch.bfloat16, device="cuda")
+    f3dc.attention(dev_bf16(qb), W, dev_bf16(kb), dev_bf16(vb), W, out, nq, nk, H, dh)
+    assert f3dc.gemm_status() == 0
+    qf, kf, vf = (synth.bf16_bits_to_f32(x) for x in (qb, kb, vb))
+    ref = orc.attention(qf[:1], kf, vf, H).astype(np.float64)  # the rows are equal
+    got = out.float().cpu().numpy().astype(np.float64)
+    assert np.isfinite(got).all()
+    assert np.max(np.abs(got - ref)) < 1e-2  # a bf16 rounding of values up to 0.7 and of P
