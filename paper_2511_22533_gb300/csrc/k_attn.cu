@@ -32,10 +32,12 @@
 // loss: P, l and O are floating point, with the same 8 exponent bits, so only
 // an overflow would be, and a ragged tile's raise whose factor underflows.  Both
 // are seen at the item's end (l above 2^64, O not finite; such a raise makes l
-// infinite).  The CTA then does its items a second time with the maximum of
+// infinite).  The CTA then does those items a second time with the maximum of
 // every key tile, m raised (O_t and l rescaled in place) when a tile's maximum
-// is 2^8 above it.  So the loop over the key tiles takes no maximum and has
-// no branch on the data.
+// is 2^8 above it, and stores the rows that asked for it alone (they stored
+// nothing before): the others keep the first pass's bits, whatever the rows of
+// their item or the CTA's other items hold.  So the loop over the key tiles takes
+// no maximum and has no branch on the data.
 // What bounds it: the softmax warps.  Per key tile of 128 x 128 scores an SM's
 // exponent unit needs 512 clocks (32 per clock) and the tensor core 512; the
 // kernel takes ~950 (4096 x 4096 x 16 heads, dh 64: 63.9 us = 1075 TFLOP/s;
@@ -72,13 +74,17 @@ struct AttnCfg {
     static constexpr int kTileBytes = 128 * kRowBytes;  // Q, K or V tile
     static constexpr uint32_t kAtom = 8 * kRowBytes;    // 8-row swizzle atom
     static constexpr uint32_t kSwz = DH == 64 ? kSwizzle128 : kSwizzle64;
-    static constexpr size_t kSmem = 1024 + kTileBytes * (4 + 2 * kKVStages) + 256;
+    static constexpr size_t kSmem = 1024 + kTileBytes * (4 + 2 * kKVStages) + 256 + 256 * 4;
     // TMEM columns: S_A S_B (fp32, 128 each) | O_A O_B (fp32, DH each) |
     // P_A P_B (bf16 pairs, 64 each)
     static constexpr uint32_t kColO = 256, kColP = 256 + 2 * DH;
     static constexpr uint32_t kTmemCols = 512;
     static_assert(kColP + 128 <= kTmemCols, "TMEM layout");
 };
+
+// A CTA's items run in windows of this many: a first pass over the window, then a
+// second one over the items in which a row asked for it (a bit for each).
+constexpr int kWindow = 32;
 
 struct Item {
     int q_row0, kv_row0, nk, h;  // q_row0: tile A's first row (B follows)
@@ -151,7 +157,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     uint64_t *drain = o_free + 2;
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
-    volatile int *redo_flag = abort_flag + 1;
+    // items of a window that run again (of windows by turns), and of each softmax
+    // thread's row the items of the window that it asked for
+    uint32_t *redo_items = tmem_holder + 2, *redo_row = tmem_holder + 4;
 
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     griddep_launch();
@@ -174,7 +182,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
         }
         mbar_init(drain, 2);
         *abort_flag = 0;
-        *redo_flag = 0;
+        redo_items[0] = redo_items[1] = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -209,26 +217,43 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
     // the previous kernel's outputs (Q / K / V) are complete
     griddep_wait();
 
-    // Every warp ends a pass over the CTA's items here, also when the kernel is
-    // aborting (each role's waits are bounded); a second pass follows if the
-    // softmax asked for one.
-    auto again = [&]() {
-        asm volatile("bar.sync 1, %0;" ::"n"(kAttnThreads) : "memory");
-        return *redo_flag != 0 && *abort_flag == 0;
+    // work item number n of this CTA, and whether a pass over the window at n0
+    // comes to it
+    auto item_of = [&](int n) { return (int)blockIdx.x + n * (int)gridDim.x; };
+    auto in_window = [&](int n, int n0) { return n < n0 + kWindow && item_of(n) < total; };
+    auto skipped = [&](int n, int pass) {
+        return pass != 0 && (redo_items[n / kWindow & 1] >> (n % kWindow) & 1) == 0;
     };
+    // Every warp ends a pass over a window here, also when the kernel is aborting
+    // (each role's waits are bounded), and all take the same next step: stop, the
+    // window's second pass, or the next window.
+    auto end_pass = [&](int &n0, int &pass, bool &stop) {
+        uint32_t any;
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n"
+                     " selp.u32 %0, 1, 0, q;\n}\n"
+                     : "=r"(any)
+                     : "r"(*abort_flag), "n"(kAttnThreads)
+                     : "memory");
+        stop = any != 0;
+        const bool again = pass == 0 && redo_items[n0 / kWindow & 1] != 0;
+        pass = again ? 1 : 0;
+        n0 += again ? 0 : kWindow;
+    };
+    bool stop = false;
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         reg_dec<kCtrlRegs>();
         uint32_t kv_it = 0, item_it = 0;
 #pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
+        for (int n0 = 0, pass = 0; !stop && item_of(n0) < total; end_pass(n0, pass, stop)) {
             if (lane == 0) {
                 bool ok = true;
 #pragma unroll 1
-                for (int w = blockIdx.x; w < total && ok; w += gridDim.x) {
+                for (int n = n0; ok && in_window(n, n0); ++n) {
+                    if (skipped(n, pass)) continue;
                     Item it = first_item;
-                    if (w != (int)blockIdx.x) decode_item(p, w, n_tiles, it);
+                    if (n) decode_item(p, item_of(n), n_tiles, it);
                     const uint32_t my_it = item_it++;
                     // Q buffer qb holds items qb, qb + 2, ...: its (my_it / 2)-th use
                     const uint32_t qb = my_it & 1, qph = (my_it >> 1) & 1;
@@ -260,7 +285,6 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                 }
             }
             __syncwarp();
-            if (!again()) break;
         }
     } else if (warp <= 2) {
         // ------------------------------------------------ MMA issuer of one query tile
@@ -287,8 +311,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             // ten warps at different places of a long kernel share.
             uint32_t g = 0, item = 0;  // S: key tile g of the CTA's run, in its item number item
 #pragma unroll 1
-            for (int pass = 0; pass < 2; ++pass) {
-                int w = (int)blockIdx.x - (int)gridDim.x;
+            for (int n0 = 0, pass = 0; !stop && item_of(n0) < total; end_pass(n0, pass, stop)) {
+                int n = n0 - 1;
                 uint32_t nkt = 0, j = 0;                // key tiles of the item, S's within it
                 bool pending = false, p_first = false;  // P V of key tile g - 1, the first of its item
                 uint32_t p_par = 0;                     // o_free's phase for that item
@@ -297,9 +321,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     if (j == nkt) {  // the next real work item
                         if (nkt) ++item;
                         nkt = j = 0;
-                        if ((w += gridDim.x) < total) {
+                        do ++n;
+                        while (in_window(n, n0) && skipped(n, pass));
+                        if (in_window(n, n0)) {
                             Item it;
-                            decode_item(p, w, n_tiles, it);
+                            decode_item(p, item_of(n), n_tiles, it);
                             nkt = __shfl_sync(0xffffffffu, (uint32_t)((it.nk + 127) / 128), 0);
                         }
                     }
@@ -339,12 +365,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     ++j;
                     ++g;
                 }
-                if (!again()) break;
             }
         }
     } else if (warp < 4) {
-        reg_dec<kCtrlRegs>();  // idle: gives its registers to the softmax warps
-        if (again()) again();
+        // gives its registers to the softmax warps; clears the next window's bits
+        reg_dec<kCtrlRegs>();
+#pragma unroll 1
+        for (int n0 = 0, pass = 0; !stop && item_of(n0) < total; end_pass(n0, pass, stop)) {
+            if (lane == 0) redo_items[(n0 / kWindow + 1) & 1] = 0;
+            __syncwarp();
+        }
     } else {
         // ------------------------------------------------ softmax warps
         reg_inc<kSoftmaxRegs>();
@@ -473,12 +503,15 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
             return true;
         };
         uint32_t g = 0;  // key tiles of this CTA's earlier items
+        uint32_t *const row_bits = redo_row + 128 * t + row;
 #pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
+        for (int n0 = 0, pass = 0; !stop && item_of(n0) < total; end_pass(n0, pass, stop)) {
+            if (pass == 0) *row_bits = 0;
 #pragma unroll 1
-            for (int w = blockIdx.x; w < total; w += gridDim.x) {
+            for (int n = n0; in_window(n, n0); ++n) {
+                if (skipped(n, pass)) continue;
                 Item it;
-                decode_item(p, w, n_tiles, it);
+                decode_item(p, item_of(n), n_tiles, it);
                 const int nk = __shfl_sync(0xffffffffu, it.nk, 0);
                 m_ref = -INFINITY;
                 l_run = 0.f;
@@ -525,21 +558,29 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
                     float zero = 0.f;
 #pragma unroll
                     for (int d = 0; d < DH; ++d) zero = fmaf(acc[d], 0.f, zero);  // NaN if any is inf or NaN
-                    if (pass == 0 && !(l_run <= 0x1p64f && zero == 0.f)) *redo_flag = 1;
-                    const float inv = 1.0f / l_run;
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.out + (size_t)orow * p.ldo + it.h * DH);
+                    // A row that asks for the second pass stores nothing now (out
+                    // may be q's buffer, whose row it needs again).
+                    const bool redo = pass == 0 && !(l_run <= 0x1p64f && zero == 0.f);
+                    if (redo) {
+                        *row_bits |= 1u << (n % kWindow);
+                        atomicOr(redo_items + (n / kWindow & 1), 1u << (n % kWindow));
+                    }
+                    if (pass == 0 ? !redo : (*row_bits >> (n % kWindow) & 1) != 0) {
+                        const float inv = 1.0f / l_run;
+                        uint4 *dst = reinterpret_cast<uint4 *>(p.out + (size_t)orow * p.ldo + it.h * DH);
 #pragma unroll
-                    for (int d = 0; d < DH; d += 8) {
-                        uint4 u;
-                        u.x = pack_bf16x2(acc[d] * inv, acc[d + 1] * inv);
-                        u.y = pack_bf16x2(acc[d + 2] * inv, acc[d + 3] * inv);
-                        u.z = pack_bf16x2(acc[d + 4] * inv, acc[d + 5] * inv);
-                        u.w = pack_bf16x2(acc[d + 6] * inv, acc[d + 7] * inv);
-                        dst[d / 8] = u;
+                        for (int d = 0; d < DH; d += 8) {
+                            uint4 u;
+                            u.x = pack_bf16x2(acc[d] * inv, acc[d + 1] * inv);
+                            u.y = pack_bf16x2(acc[d + 2] * inv, acc[d + 3] * inv);
+                            u.z = pack_bf16x2(acc[d + 4] * inv, acc[d + 5] * inv);
+                            u.w = pack_bf16x2(acc[d + 6] * inv, acc[d + 7] * inv);
+                            dst[d / 8] = u;
+                        }
                     }
                 }
+                __syncwarp();
             }
-            if (!again()) break;
         }
     }
     __syncthreads();

@@ -188,3 +188,86 @@ def test_attention_ragged_last_tile_far_above_the_first(orc, nq, nk, H, dh, midd
     got = out.float().cpu().numpy().astype(np.float64)
     assert np.isfinite(got).all()
     assert np.max(np.abs(got - ref)) < 1e-2  # a bf16 rounding of values up to 0.7 and of P
+
+
+def _bits(t):
+    return t.view(torch.int16).cpu().numpy()
+
+
+@pytest.mark.parametrize("nq,nk,H,dh", [(2700, 900, 16, 64), (4096, 700, 16, 64), (4096, 700, 16, 32)])
+@pytest.mark.parametrize("which", ["all", "one"])
+def test_attention_second_pass_over_several_items(orc, nq, nk, H, dh, which):
+    # 176 and 256 (pair, head) items on 152 SMs: CTAs with one item and CTAs
+    # with two, whose second pass starts at other K/V stages, Q buffers and
+    # barrier phases than the first did.  "all": every row's scores rise by
+    # 2^90 after the first key tile, so every item runs twice.  "one": a single
+    # row of one head does, in the second item of its CTA (152 + 3), and only
+    # that item does.  Written over the queries the result is the same.
+    g = np.random.default_rng(nq + nk + dh)
+    W = H * dh
+    u = np.where(g.random((H, dh)) < 0.5, -1.0, 1.0)
+    unit = 1.0 / (np.sqrt(dh) * np.log2(np.e))
+    a = np.zeros(nk)
+    a[200:300] = 90.0 * unit
+    a[nk - 30:] = 80.0 * unit
+    k = (np.einsum("j,hd->jhd", a, u) + 0.02 * g.standard_normal((nk, H, dh))).reshape(nk, W)
+    v = g.standard_normal((nk, W))
+    # strength 0.01: scores up to 0.9
+    c = np.full((nq, H), 1.0 if which == "all" else 0.01)
+    item = 152 + 3
+    row, head = 256 * (item // H) + 5, item % H
+    c[row, head] = 1.0
+    q = np.einsum("rh,hd->rhd", c, u).reshape(nq, W)
+    qb, kb, vb = (synth.f32_to_bf16_bits(x.astype(np.float32)) for x in (q, k, v))
+    out = torch.zeros((nq, W), dtype=torch.bfloat16, device="cuda")
+    f3dc.attention(dev_bf16(qb), W, dev_bf16(kb), dev_bf16(vb), W, out, nq, nk, H, dh)
+    assert f3dc.gemm_status() == 0
+    qd = dev_bf16(qb)
+    f3dc.attention(qd, W, dev_bf16(kb), dev_bf16(vb), W, qd, nq, nk, H, dh)
+    assert f3dc.gemm_status() == 0 and torch.equal(qd, out)
+    rows = np.unique(np.concatenate([[0, 127, 128, 255, 256, row - 1, row, row + 1, nq - 1], g.integers(0, nq, 40)]))
+    qf, kf, vf = (synth.bf16_bits_to_f32(x) for x in (qb, kb, vb))
+    ref = orc.attention(qf[rows], kf, vf, H).astype(np.float64)
+    got = out.float().cpu().numpy()
+    assert np.isfinite(got).all()
+    assert rel_l2(got[rows], ref) < 1e-2
+    assert np.max(np.abs(got[rows] - ref)) < 2e-2
+
+
+@pytest.mark.parametrize("nq,nk,H,dh", [(1280, 900, 16, 64), (4096, 700, 16, 32)])
+@pytest.mark.parametrize("bad", ["nan", "far"])
+def test_attention_rows_do_not_depend_on_others_second_pass(nq, nk, H, dh, bad):
+    # a row whose scores are NaN, or 2^90 above those of the first key tile,
+    # wants its item done again; every other row keeps its bits (but for the 32
+    # rows of its warp and head, which raise their reference together), those of
+    # its item, of its CTA's other items and of the other heads.  Key strengths
+    # rise by 2^10 and 2^20, so that running maxima would take another
+    # reference than the first key tile's.
+    g = np.random.default_rng(nq + nk + dh)
+    W = H * dh
+    u = np.where(g.random((H, dh)) < 0.5, -1.0, 1.0)
+    unit = 1.0 / (np.sqrt(dh) * np.log2(np.e))
+    a = np.zeros(nk)
+    a[150:256] = 10.3 * unit
+    a[256:400] = 20.7 * unit
+    k = (np.einsum("j,hd->jhd", a, u) + 0.1 * g.standard_normal((nk, H, dh))).reshape(nk, W)
+    v = dev_bf16(synth.f32_to_bf16_bits(g.standard_normal((nk, W)).astype(np.float32)))
+    q = (np.broadcast_to(u, (nq, H, dh)) + 0.1 * g.standard_normal((nq, H, dh))).astype(np.float32)
+    row, head = 300, 3
+    kd = dev_bf16(synth.f32_to_bf16_bits(k.astype(np.float32)))
+
+    def run(q):
+        out = torch.zeros((nq, W), dtype=torch.bfloat16, device="cuda")
+        f3dc.attention(dev_bf16(synth.f32_to_bf16_bits(q.reshape(nq, W))), W, kd, v, W, out, nq, nk, H, dh)
+        assert f3dc.gemm_status() == 0
+        return _bits(out).reshape(nq, H, dh)
+
+    clean = run(q)
+    q2 = q.copy()
+    q2[row, head] = np.nan if bad == "nan" else 5.0 * u[head]
+    got = run(q2)
+    changed = np.any(got != clean, axis=2)
+    changed[row // 32 * 32:row // 32 * 32 + 32, head] = False
+    assert not changed.any(), np.argwhere(changed)[:5]
+    if bad == "nan":
+        assert np.isnan(synth.bf16_bits_to_f32(got[row, head].view(np.uint16))).all()

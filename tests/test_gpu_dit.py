@@ -10,7 +10,7 @@ import torch
 
 from gpu_helpers import (VEL_MAX_ABS, VEL_REL_L2, assert_clean, dev_f32, dev_i32, dev_u16, handle_for, host_u16,
                          max_abs, rel_l2, stored_vel_excess)
-from paper_2511_22533_gb300 import synth
+from paper_2511_22533_gb300 import f3dc, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -395,3 +395,69 @@ def test_step_batch64_32cubed_merge(orc):
         np.testing.assert_array_equal(S_gpu[b], S_o)
         assert np.isfinite(synth.bf16_bits_to_f32(vt[b])).all()
     h.close()
+
+
+def _steep(blob, shape, gain, cross=1.0):
+    # query and key norms' gains: scaled self-attention scores of standard
+    # deviation 1.44 gain^2 (log2 units); cross-attention scores `cross` times as large
+    for l in range(shape.blocks):
+        synth.set_weight(blob, shape, "qn_g", l, np.float32(gain))
+        synth.set_weight(blob, shape, "kn_g", l, np.float32(gain))
+        synth.set_weight(blob, shape, "cq_w", l, cross * synth.weight_view(blob, shape, "cq_w", l))
+    return blob
+
+
+def test_forward_sample_does_not_depend_on_its_neighbour():
+    # 32 samples of 512 tokens and 4 heads: 256 (pair, head) items on 152 SMs, so
+    # a CTA serves several samples.  NaN in one of them asks for a second pass,
+    # with another reference where scores are this spread; the others keep
+    # their bits.
+    B = 32
+    blob = _steep(synth.weights_blob(TINY, 0), TINY, 3.0)
+    h = f3dc.Handle(f3dc.config_for(TINY, B), dev_u16(blob))
+    h.set_cond(dev_u16(synth.cond_tokens(TINY, B, 0)), B)
+    S = synth.latents(TINY, B, 0)
+    lists = [np.arange(512)] * B
+    clean = _forward_gpu(h, 0.5, S, lists)
+    S[0, 100] = np.nan
+    got = _forward_gpu(h, 0.5, S, lists)
+    assert np.isnan(got[0]).any()
+    for b in range(1, B):
+        np.testing.assert_array_equal(got[b].view(np.uint32), clean[b].view(np.uint32), err_msg=f"sample {b}")
+    h.close()
+
+
+@pytest.mark.parametrize("gain,cross", [(8.0, 1.0), (1.0, 60.0)])
+def test_forward_attention_second_pass_in_a_model(orc, gain, cross):
+    # scores of standard deviation 92 (self) or about 87 (cross) log2 units: many
+    # rows find a key 2^64 above their first key tile's, so the pair kernel (all
+    # of f3dc_forward's attention) runs a second pass over the plan's pairs.  A
+    # sampling run of one step (t 1 to 0) of one sample takes the one-tile kernel
+    # (16 items), which keeps running maxima: the same velocity, up to the
+    # rounding of P and the velocity's to bf16.  One block, and no self-attention
+    # output before the steep cross-attention: the two kernels' results differ by
+    # a bf16 rounding (2^-9), which in the query moves a row's largest score
+    # (3 standard deviations, 260) by 0.5, its weights by 40 %.
+    shape = synth.ModelShape(8, 8, 128, 1, 4, 4, 300, 128, 1, 64)
+    B = 3
+    blob = _steep(synth.weights_blob(shape, 0), shape, gain, cross)
+    if cross > 1.0:
+        synth.set_weight(blob, shape, "o_w", 0, np.float32(0.0))
+    blob = dev_u16(blob)
+    cond, S = synth.cond_tokens(shape, B, 0), synth.latents(shape, B, 0)
+    h = f3dc.Handle(f3dc.config_for(shape, B), blob)
+    h.set_cond(dev_u16(cond), B)
+    got = _forward_gpu(h, 1.0, S, [np.arange(512)] * B)
+    assert_clean(h)
+    h.close()
+    one = f3dc.Handle(f3dc.config_for(shape, 1), blob)
+    for b in range(B):
+        S1 = dev_f32(S[b:b + 1])
+        one.sample(S1, dev_u16(cond[b:b + 1]), 1, sigma_override=[0.0], quota_schedule=np.zeros((1, 1), np.int32))
+        torch.cuda.synchronize()
+        ref = S[b] - S1.cpu().numpy()[0]
+        assert np.isfinite(got[b]).all()
+        assert stored_vel_excess(got[b], ref) < 0, (b, max_abs(got[b], ref))
+        assert rel_l2(got[b], ref) < VEL_REL_L2, (b, rel_l2(got[b], ref))
+    assert_clean(one)
+    one.close()
