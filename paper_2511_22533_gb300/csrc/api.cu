@@ -1463,13 +1463,13 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     const int tiles = p.m_tiles * (N / bn);
     const int epi = epilogue == F3DC_EPI_BIAS ? kEpiBias : (epilogue == F3DC_EPI_GELU ? kEpiGelu : kEpiResid);
     cudaStream_t s = (cudaStream_t)stream;
-    const bool split = gemm_split_count(tiles, gemm_grid(tiles, sms), K / 64, sms, true) > 1;
+    const int splits = gemm_split_count(tiles, gemm_grid(tiles, sms), K / 64, sms, true);
     if (pair) {
-        p.pieces = split;
+        p.piece_kb = gemm_piece_kb(K, splits);
         CK(launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s));
         return F3DC_OK;
     }
-    if (!split) {
+    if (splits == 1) {
         CK(launch_gemm(&ta, &tb, p, epi, bn, tiles < sms ? tiles : sms, s));
         return F3DC_OK;
     }

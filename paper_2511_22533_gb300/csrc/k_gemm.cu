@@ -108,25 +108,22 @@ struct TmemSrc {
     }
 };
 
-// Adds accumulators 1 .. n - 1 (bn TMEM columns apart) to accumulator 0 in
+// Adds n accumulators, bn TMEM columns apart from `add` on, to the one at `acc` in
 // order, in the 32-column chunks k0, k0 + kstep, ... of this warp's lanes.
-F3DC_DEV void sum_accumulators(uint32_t tbase, int bn, int n, int k0, int kstep)
+F3DC_DEV void add_accumulators(uint32_t acc, uint32_t add, int bn, int n, int k0, int kstep)
 {
 #pragma unroll 1
     for (int c0 = 32 * k0; c0 < bn; c0 += 32 * kstep) {
-        float v[32];
-        TmemSrc{tbase}(c0, v);
+        uint32_t r[32], w[32];
+        tmem_ld32(acc + c0, r);
 #pragma unroll 1
-        for (int a = 1; a < n; ++a) {
-            float w[32];
-            TmemSrc{tbase + (uint32_t)(a * bn)}(c0, w);
+        for (int a = 0; a < n; ++a) {
+            tmem_ld32(add + (uint32_t)(a * bn) + c0, w);
+            tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += w[j];
+            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(w[j]));
         }
-        uint32_t r[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(v[j]);
-        tmem_st32(tbase + c0, r);
+        tmem_st32(acc + c0, r);
     }
     tmem_wait_st();
 }
@@ -614,8 +611,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 //   full[s]  (even CTA): both CTAs' TMA bytes of stage s (the even CTA's
 //            producer posts the expected count)
 //   empty[s] (both):     stage s consumed (multicast MMA commit)
-//   accf[b]  (both):     accumulator buffer b complete (multicast commit)
-//   acce[b]  (even CTA): buffer b read by the epilogue warps of both CTAs
+//   accf[b]  (both):     accumulator b complete (multicast commit)
+//   acce[b]  (even CTA): accumulator b read by the epilogue warps of both CTAs
 // A stage holds 128 K: two 64-column boxes per operand row block, each a
 // 128B-swizzled K-major region of its own ([half][rows][128 B]).
 constexpr int kPairBK = 128;
@@ -675,7 +672,18 @@ struct PairUnits {
     }
 };
 
-template <int EPI>
+// kPieces: a unit's K is summed in pieces of at most p.piece_kb stages, each in an
+// accumulator of its own, added in order in fp32.  The tensor core truncates as it
+// accumulates, so the error of a sum grows with its length (of random signs, 4096:
+// 3.2e-6 relative, 1024: 1e-6, 256: 2.4e-7).  TMEM holds 512 / bn accumulators: the first takes the
+// sum, and where there are more pieces than accumulators the others take turns,
+// the epilogue warps adding one while the next is computed.  A kernel of its own:
+// the steps' launches sum the whole K and start with a cold instruction cache.
+// Error (2-norm, positive products) and time of one sum of the whole K, of pieces,
+// and of the single-CTA kernel's split K: 1 x 1024 x 4096 9e-6 (four accumulators
+// without turns: 2.2e-6, 14.7 us), 16 pieces 3.8e-7, 20 us, split K 3.8e-7, 29.5 us;
+// 1229 x 1024 x 4096 four pieces 2.2e-6, 17.3 us, split K 3.0e-6, 30.8 us.
+template <int EPI, bool kPieces>
 __global__ void __launch_bounds__(kPairThreads, 1)
     k_gemm_pair(const __grid_constant__ CUtensorMap tma, const __grid_constant__ GemmPairB tmb,
                 const __grid_constant__ CUtensorMap tmo, const GemmParams p)
@@ -687,7 +695,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     uint8_t *sb = smem + S * kPairAStage;
     uint8_t *so = sb + S * kPairBStage;
     uint64_t *bars = reinterpret_cast<uint64_t *>(so + 2 * kPairOutBufs * kOutChunkBytes);
-    uint64_t *full = bars, *empty = bars + S, *accf = bars + 2 * S, *acce = accf + 2, *drain = acce + 2;
+    constexpr int kAccs = kPieces ? 8 : 2;
+    uint64_t *full = bars, *empty = bars + S, *accf = bars + 2 * S, *acce = accf + kAccs, *drain = acce + kAccs;
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
 
@@ -709,10 +718,11 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
-        mbar_init(&accf[0], 1);
-        mbar_init(&accf[1], 1);
-        mbar_init(&acce[0], 16);  // eight epilogue warps in each CTA
-        mbar_init(&acce[1], 16);
+#pragma unroll
+        for (int b = 0; b < kAccs; ++b) {
+            mbar_init(&accf[b], 1);
+            mbar_init(&acce[b], 16);  // eight epilogue warps in each CTA
+        }
         mbar_init(drain, 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -753,14 +763,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                              mapa_shared(smem_u32(full), 0) + 8u * (uint32_t)s);
     }
     griddep_wait();  // the previous kernel's outputs (A, x) are complete
-    // The tensor core truncates as it accumulates, so the error of a sum grows
-    // with its length (4096: 3.2e-6 relative, 1024: 7e-7).  A long K is summed
-    // in pieces where the second TMEM buffer is not needed for a next unit:
-    // as many accumulators as fit in TMEM, added in fp32 by the epilogue.  Only
-    // for fp32 results: a bf16 one rounds at 2^-9.
-    const int chunks = EPI == kEpiResid && p.pieces && U.total <= ncl ? (int)kPairTmemCols / (U.full ? 256 : 256 / U.sub) : 1;
-    const uint32_t chunk_kb = (uint32_t)((kb_n + chunks - 1) / chunks);
-    const int n_acc = (kb_n + (int)chunk_kb - 1) / (int)chunk_kb;
+    // of a unit bn columns wide: the stages that fill TMEM's accumulators once, its
+    // pieces' length, whether there are more pieces than accumulators (these then
+    // take turns; otherwise one commit and one wait do), and the accumulator after b
+    auto even_kb = [&](int bn) { return (kb_n * bn + (int)kPairTmemCols - 1) / (int)kPairTmemCols; };
+    auto piece_kb = [&](int bn) { return min(p.piece_kb, even_kb(bn)); };
+    auto by_turns = [&](int bn) { return p.piece_kb < even_kb(bn); };
+    auto next_acc = [&](int b, int bn) { return (b + 1) * bn < (int)kPairTmemCols ? b + 1 : 1; };
     const uint32_t full_c = mapa_shared(smem_u32(full), 0);  // the even CTA's full[0]
     const uint32_t acce_c = mapa_shared(smem_u32(acce), 0);
 
@@ -802,20 +811,23 @@ __global__ void __launch_bounds__(kPairThreads, 1)
             const uint64_t b_desc0 = make_sdesc(smem_u32(sb), 16, 1024, kSwizzle128);
             int s = 0, it = 0;
             uint32_t ph = 0;
+            uint32_t used = 0;  // kPieces: each accumulator's phase
             bool ok = true;
             bool ready = warp_all(mbar_test(&full[0], 0));
+            auto acc_free = [&](int b, uint32_t par) {
+                return warp_all(mbar_test(&acce[b], par)) || warp_all(mbar_wait(&acce[b], par, abort_flag, p.err));
+            };
 #pragma unroll 1
             for (int t = cl; t < U.total && ok; t += ncl, ++it) {
                 const int bn = t < U.full ? 256 : 256 / U.sub;
                 const uint32_t idesc = make_idesc_bf16(256, bn, 0, 0);
                 const uint64_t b_half = (uint64_t)(bn / 2 * 128) >> 4;  // from a stage's first 64 K of B to the second
-                const int buf = it & 1;
-                const uint32_t aph = (it >> 1) & 1;
-                if (!warp_all(mbar_test(&acce[buf], aph ^ 1)) &&
-                    !warp_all(mbar_wait(&acce[buf], aph ^ 1, abort_flag, p.err)))
-                    break;
-                uint32_t d = tmem + buf * 256, left = chunk_kb;
+                int buf = kPieces ? 0 : it & 1;
+                if (!acc_free(buf, (kPieces ? used : (it >> 1) & 1) & 1 ^ 1)) break;
+                uint32_t d = tmem + (kPieces ? 0 : buf * 256);
+                int left = kPieces ? piece_kb(bn) : 0;
                 bool first = true;
+                const bool turns = kPieces && by_turns(bn);
 #pragma unroll 1
                 for (int kb = 0; kb < kb_n; ++kb) {
                     if (!ready && !warp_all(mbar_wait(&full[s], ph, abort_flag, p.err))) {
@@ -830,15 +842,28 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     const uint64_t bd = b_desc0 + (uint64_t)s * (kPairBStage >> 4);
                     mma_bf16_pair_128k(d, ad, bd, kPairHalf >> 4, b_half, idesc, !first);
                     mma_commit_pair_mc_elect(&empty[s], 3);
-                    first = --left == 0;
-                    if (first) {  // the next accumulator
-                        d += bn;
-                        left = chunk_kb;
+                    first = false;
+                    if (kPieces && --left == 0 && kb + 1 < kb_n) {  // the next piece
+                        const int next = next_acc(buf, bn);
+                        if (turns) {
+                            mma_commit_pair_mc_elect(&accf[buf], 3);
+                            used ^= 1u << buf;
+                            if (!acc_free(next, (used >> next & 1) ^ 1)) {
+                                ok = false;
+                                break;
+                            }
+                        }
+                        buf = next;
+                        d = tmem + (uint32_t)(buf * bn);
+                        left = piece_kb(bn);
+                        first = true;
                     }
                     s = s_next;
                     ph = ph_next;
                 }
+                if (kPieces && !turns) buf = 0;
                 if (ok) mma_commit_pair_mc_elect(&accf[buf], 3);
+                used ^= 1u << buf;
             }
         }
     } else {
@@ -846,35 +871,64 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         const int row = q * 32 + lane;
         const int grp = (warp - 2) >> 2;
         OutStage o{so + grp * kPairOutBufs * kOutChunkBytes, &tmo, row, 0, kPairOutBufs, 3 + grp, 64 + 128 * grp};
-        int it = 0;
-#pragma unroll 1
-        for (int t = cl; t < U.total; t += ncl, ++it) {
-            const int buf = it & 1;
-            const uint32_t aph = (it >> 1) & 1;
-            int m, n0, bn;
-            U.decode(t, m, n0, bn);
-            ColOps first;
-            if constexpr (EPI != kEpiQKNorm) load_colops<EPI>(p, n0 + 32 * grp, first);
-            const uint32_t got = mbar_wait(&accf[buf], aph, abort_flag, p.err) ? 1u : 0u;
+        // the same answer for the group's four warps, whose staging waits for all
+        auto all_warps = [&](bool ok) {
             uint32_t all;
             asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, 128, p;\n"
                          " selp.u32 %0, 1, 0, q;\n}\n"
                          : "=r"(all)
-                         : "r"(got), "r"(o.bar)
+                         : "r"(ok ? 1u : 0u), "r"(o.bar)
                          : "memory");
-            if (!all) break;
-            tc_fence_after();
+            return all != 0;
+        };
+        auto acc_read = [&](int b) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(acce_c + 8u * (uint32_t)b);
+        };
+        const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
+        int it = 0;
+        uint32_t used = 0;  // kPieces: each accumulator's phase
+#pragma unroll 1
+        for (int t = cl; t < U.total; t += ncl, ++it) {
+            int m, n0, bn;
+            U.decode(t, m, n0, bn);
+            ColOps first;
+            if constexpr (EPI != kEpiQKNorm) load_colops<EPI>(p, n0 + 32 * grp, first);
             const int m0 = m * 256 + (int)rank * 128;
             // the odd CTA's rows of the last pair lie beyond the plan when
             // the tile count is odd: computed, not stored
-            if (m0 < m_tiles * 128) {
-                const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256);
-                if (EPI == kEpiResid && n_acc > 1) sum_accumulators(acc, bn, n_acc, grp, 2);
-                epilogue_tile<EPI>(p, TmemSrc{acc}, o, m0, n0, bn, grp, 2, &first);
+            const bool rows = m0 < m_tiles * 128;
+            if constexpr (kPieces) {
+                bool ok = warp_all(mbar_wait(&accf[0], used & 1, abort_flag, p.err));
+                used ^= 1;
+                tc_fence_after();
+                // the pieces after the first: all at once, or one by one as they
+                // are computed where they take turns
+                const bool turns = by_turns(bn);
+                int buf = 1, left = (kb_n - 1) / piece_kb(bn);
+                const int step = turns ? 1 : left;
+#pragma unroll 1
+                for (; ok && left > 0; left -= step) {
+                    if (turns) {
+                        ok = warp_all(mbar_wait(&accf[buf], used >> buf & 1, abort_flag, p.err));
+                        used ^= 1u << buf;
+                        tc_fence_after();
+                    }
+                    if (rows) add_accumulators(lanes, lanes + (uint32_t)(buf * bn), bn, step, grp, 2);
+                    if (turns) acc_read(buf);
+                    buf = next_acc(buf, bn);
+                }
+                if (!all_warps(ok)) break;
+                if (rows) epilogue_tile<EPI>(p, TmemSrc{lanes}, o, m0, n0, bn, grp, 2, &first);
+                acc_read(0);
+            } else {
+                const int buf = it & 1;
+                if (!all_warps(mbar_wait(&accf[buf], (it >> 1) & 1, abort_flag, p.err))) break;
+                tc_fence_after();
+                if (rows) epilogue_tile<EPI>(p, TmemSrc{lanes + (uint32_t)(buf * 256)}, o, m0, n0, bn, grp, 2, &first);
+                acc_read(buf);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(acce_c + 8u * (uint32_t)buf);
         }
         if ((int)threadIdx.x == o.issuer) bulk_wait_all();
     }
@@ -896,7 +950,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
 }
 
-template <int EPI>
+template <int EPI, bool kPieces>
 cudaError_t launch_pair_one(const CUtensorMap *ta, const GemmPairB *tb, const CUtensorMap *to, const GemmParams &p,
                             int max_units, cudaStream_t s)
 {
@@ -908,7 +962,7 @@ cudaError_t launch_pair_one(const CUtensorMap *ta, const GemmPairB *tb, const CU
     if (e != cudaSuccess) return e;
     int max_clusters = max_clusters_of[dev & 63].load(std::memory_order_acquire);
     if (!max_clusters) {
-        e = cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+        e = cudaFuncSetAttribute(k_gemm_pair<EPI, kPieces>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2);
@@ -922,7 +976,7 @@ cudaError_t launch_pair_one(const CUtensorMap *ta, const GemmPairB *tb, const CU
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k_gemm_pair<EPI>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&n, k_gemm_pair<EPI, kPieces>, &cfg);
         if (e != cudaSuccess) return e;
         if (n < 1) return cudaErrorInvalidConfiguration;
         max_clusters = n;
@@ -943,7 +997,7 @@ cudaError_t launch_pair_one(const CUtensorMap *ta, const GemmPairB *tb, const CU
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, k_gemm_pair<EPI>, *ta, *tb, *to, p);
+    e = cudaLaunchKernelEx(&cfg, k_gemm_pair<EPI, kPieces>, *ta, *tb, *to, p);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -1056,11 +1110,19 @@ cudaError_t launch_gemm_pair(const CUtensorMap *ta, const GemmPairB *tb, const G
     CUtensorMap to;
     if (!make_tmap_out(&to, p.out, (uint64_t)p.M, (uint64_t)p.N, (uint64_t)p.ldo, epi == kEpiResid))
         return cudaErrorInvalidValue;
+    const bool pieces = p.piece_kb > 0;
     switch (epi) {
-    case kEpiBias: return launch_pair_one<kEpiBias>(ta, tb, &to, p, max_units, s);
-    case kEpiGelu: return launch_pair_one<kEpiGelu>(ta, tb, &to, p, max_units, s);
-    case kEpiResid: return launch_pair_one<kEpiResid>(ta, tb, &to, p, max_units, s);
-    case kEpiQKNorm: return launch_pair_one<kEpiQKNorm>(ta, tb, &to, p, max_units, s);
+    case kEpiBias:
+        return pieces ? launch_pair_one<kEpiBias, true>(ta, tb, &to, p, max_units, s)
+                      : launch_pair_one<kEpiBias, false>(ta, tb, &to, p, max_units, s);
+    case kEpiGelu:
+        return pieces ? launch_pair_one<kEpiGelu, true>(ta, tb, &to, p, max_units, s)
+                      : launch_pair_one<kEpiGelu, false>(ta, tb, &to, p, max_units, s);
+    case kEpiResid:
+        return pieces ? launch_pair_one<kEpiResid, true>(ta, tb, &to, p, max_units, s)
+                      : launch_pair_one<kEpiResid, false>(ta, tb, &to, p, max_units, s);
+    case kEpiQKNorm:
+        return pieces ? cudaErrorInvalidValue : launch_pair_one<kEpiQKNorm, false>(ta, tb, &to, p, max_units, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -166,10 +166,9 @@ struct GemmParams {
     float *ws;
     int32_t *counters;
     int ws_units;             // partial tiles the workspace holds
-    // CTA pairs, RESID: sum a long K in pieces (several accumulators, added in
-    // fp32) where TMEM has room; set for the problems that launch_gemm would
-    // split, whose shorter sums are the more precise ones
-    int pieces;
+    // CTA pairs: longest sum in one accumulator, in stages of 128 K (0: the whole
+    // K), see gemm_piece_kb
+    int piece_kb;
     // fault injection (tests of the failure path; 0 in normal use): the
     // split-K arrival wait expects split_extra arrivals beyond the splits
     // that exist, and gives up after split_wait_ns (0: kWaitLimitNs)
@@ -200,9 +199,13 @@ struct GemmPairB {
 bool make_tmap_pair(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, uint32_t box_rows);
 bool make_tmap_pair_b(GemmPairB *maps, const void *base, uint64_t rows, uint64_t K);
 // f3dc_gemm's rule: pairs for every shape they can compute.  At 1229 x 1024 x
-// 4096 they take 16.4 us against 29.9 us for the single-CTA kernel with split K,
-// at 1 x 1024 x 4096 14.1 us against 28.8 us.
+// 4096 they take 17.3 us against 30.8 us for the single-CTA kernel with split K,
+// at 1 x 1024 x 4096 20 us against 29.5 us.
 inline bool gemm_on_pairs(int N, int K) { return N % 256 == 0 && K % 128 == 0; }
+// Where launch_gemm would split K, its partial sums are shorter, and so more precise,
+// than one sum of the whole K: the pairs then sum pieces no longer than one of its
+// `splits` (which has at least four blocks of 64).
+inline int gemm_piece_kb(int K, int splits) { return splits > 1 ? (K / 64 + splits - 1) / splits / 2 : 0; }
 cudaError_t launch_gemm_pair(const CUtensorMap *ta, const GemmPairB *tb, const GemmParams &p, int epi, int max_units,
                              cudaStream_t s);
 size_t gemm_smem_bytes(int bn);

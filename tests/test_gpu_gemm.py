@@ -137,3 +137,46 @@ def test_gemm_pair_units(M, N, K, epi):
         assert ((out.double() - ref).norm() / ref.norm()).item() < 2e-6
         assert (out.double() - ref).abs().max().item() < 1e-4
     assert f3dc.gemm_status() == 0
+
+
+def _split_length(M, N, K):
+    """K per partial sum where the library splits K over CTAs (its rule, restated)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bn = 256 if N % 256 == 0 else (128 if N % 128 == 0 else 64)
+    tiles, kb = -(-M // 128) * (N // bn), K // 64
+    sp = min(sms // tiles, kb // 4, 16) if 2 * tiles <= sms and kb >= 32 else 1
+    return 64 * -(-kb // max(sp, 1))
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1024, 4096), (64, 1024, 4096), (128, 1024, 2048), (77, 512, 5120),
+                                   (300, 1024, 4096), (500, 2048, 2176), (384, 6400, 2048), (129, 256, 8192)])
+@pytest.mark.parametrize("epi", [f3dc.EPI_BIAS, f3dc.EPI_GELU, f3dc.EPI_RESID])
+def test_gemm_long_sums_in_pieces(M, N, K, epi):
+    # few tiles and a long K: sums in pieces no longer than split K's, in units of
+    # 64, 128 and 256 columns, with fewer and more pieces than TMEM holds
+    # accumulators (2 to 16), and a last piece that is shorter.  Positive
+    # products, so that truncation adds up: a step of 16 K loses 2^-24 of the sum
+    # so far on average (up to 2^-23), a piece of L (L / 32) 2^-24 = 1.9e-9 L of
+    # itself, the fp32 sum of the pieces about 1e-7.  A bias close to -sum shows
+    # the same in a bf16 result.
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.randn(M, K, generator=g, device="cuda").abs().bfloat16()
+    Bw = torch.randn(N, K, generator=g, device="cuda").abs().bfloat16()
+    y = A.double() @ Bw.double().T
+    rel = 2.2e-9 * _split_length(M, N, K) + 1.5e-7
+    if epi == f3dc.EPI_RESID:
+        out = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+        f3dc.gemm(A, Bw, None, None, out, M, N, K, epi)
+        assert ((out.double() - y).norm() / y.norm()).item() <= rel
+        assert ((out.double() - y) / y).abs().max().item() <= 2 * rel
+    else:
+        bias = (-y.mean(0)).bfloat16()
+        out = torch.full((M, N), 7.0, dtype=torch.bfloat16, device="cuda")
+        f3dc.gemm(A, Bw, bias, None, out, M, N, K, epi)
+        ref = y + bias.double()
+        slack = 2 * rel * y.max()
+        if epi == f3dc.EPI_GELU:
+            # slope up to 1.13; tanh.approx is off by 2^-11, times |x| / 2 where that matters (|x| < 4)
+            ref, slack = torch.nn.functional.gelu(ref, approximate="tanh"), 1.13 * slack + 1e-3
+        assert torch.all((out.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + slack)
+    assert f3dc.gemm_status() == 0
