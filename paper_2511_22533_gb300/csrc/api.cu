@@ -1440,8 +1440,10 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int m_tiles = (M + kTileRows - 1) / kTileRows;
+    const int tiles = m_tiles * (N / bn);
+    const int splits = gemm_split_count(tiles, gemm_grid(tiles, sms), K / 64, sms, true);
     // the injected missing arrival is the split-K kernel's
-    const bool pair = gemm_on_pairs(N, K) && fault_injection().gemm_missing_arrivals == 0;
+    const bool pair = gemm_on_pairs(M, N, K, splits) && fault_injection().gemm_missing_arrivals == 0;
     CUtensorMap ta, tb;
     GemmPairB tbp;
     if (!(pair ? make_tmap_pair(&ta, A, M, K, 128) && make_tmap_pair_b(&tbp, B, N, K)
@@ -1460,10 +1462,8 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     // a bounded wait that runs out is recorded here (read by f3dc_gemm_status)
     p.err = gemm_status_word();
     if (!p.err) return fail(nullptr, F3DC_ERR_CUDA, "cannot resolve the GEMM status word");
-    const int tiles = p.m_tiles * (N / bn);
     const int epi = epilogue == F3DC_EPI_BIAS ? kEpiBias : (epilogue == F3DC_EPI_GELU ? kEpiGelu : kEpiResid);
     cudaStream_t s = (cudaStream_t)stream;
-    const int splits = gemm_split_count(tiles, gemm_grid(tiles, sms), K / 64, sms, true);
     if (pair) {
         p.piece_kb = gemm_piece_kb(K, splits);
         CK(launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s));

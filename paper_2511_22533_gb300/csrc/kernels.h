@@ -198,10 +198,21 @@ struct GemmPairB {
 };
 bool make_tmap_pair(CUtensorMap *map, const void *base, uint64_t rows, uint64_t K, uint32_t box_rows);
 bool make_tmap_pair_b(GemmPairB *maps, const void *base, uint64_t rows, uint64_t K);
-// f3dc_gemm's rule: pairs for every shape they can compute.  At 1229 x 1024 x
-// 4096 they take 17.3 us against 30.8 us for the single-CTA kernel with split K,
-// at 1 x 1024 x 4096 20 us against 29.5 us.
-inline bool gemm_on_pairs(int N, int K) { return N % 256 == 0 && K % 128 == 0; }
+// f3dc_gemm's rule: pairs for every shape they can compute, but for a very long K
+// that launch_gemm would split (`splits` > 1): a pair runs through the whole K, 0.3 us
+// per 128, so the few clusters of such a launch are its time, and split K wins
+// from there on, earlier with one row tile, where half of every pair's rows are
+// empty.  Residual, pairs / split K, us:
+//   M x N           K 4096       6144         8192         12288
+//   1 x 256         20.1 / 26.6  21.7 / 26.7  26.1 / 26.8  35 / 28.8
+//   128 x 12800     33.0 / 42.8  48.8 / 51.5  65.7 / 59.5  94 / 74
+//   300 x 1024      16.0 / 24.7  20.8 / 26.7  25.7 / 27.0  35 / 28.8
+//   1229 x 1024     17.3 / 30.8  22.2 / 32.9  27.5 / 36.9  48 / 45.3
+// and 4 x 256 x 65536 158 / 42.
+inline bool gemm_on_pairs(int M, int N, int K, int splits)
+{
+    return N % 256 == 0 && K % 128 == 0 && (splits == 1 || K <= (M > kTileRows ? 8192 : 6144));
+}
 // Where launch_gemm would split K, its partial sums are shorter, and so more precise,
 // than one sum of the whole K: the pairs then sum pieces no longer than one of its
 // `splits` (which has at least four blocks of 64).

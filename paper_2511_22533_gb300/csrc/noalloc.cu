@@ -111,7 +111,7 @@ extern "C" f3dc_status f3dc_gemm_noalloc(const void *A, const void *B, const voi
     const int tiles = m_tiles * (N / bn);
     const int grid = gemm_grid(tiles, sms);
     const int splits = gemm_split_count(tiles, grid, K / 64, sms, true);
-    const bool pair = gemm_on_pairs(N, K);
+    const bool pair = gemm_on_pairs(M, N, K, splits);
     const size_t need = !pair && splits > 1 ? gemm_ws_bytes(bn, tiles * splits) : 0;
     if (need > kPartialBytes)
         return fail(F3DC_ERR_INVALID_ARG, "this problem needs " + std::to_string(need) +

@@ -2,6 +2,8 @@
 fp64-accumulated nn.Linear (Supp. Sec. F projections), on sampled output
 rows at the transformer's shapes (active-token counts 1229 / 4096, widths
 1024 / 3072 / 4096, K 1024 / 4096) and on ragged small cases."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -180,3 +182,27 @@ def test_gemm_long_sums_in_pieces(M, N, K, epi):
             ref, slack = torch.nn.functional.gelu(ref, approximate="tanh"), 1.13 * slack + 1e-3
         assert torch.all((out.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + slack)
     assert f3dc.gemm_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K,nodes", [
+    (1, 256, 6144, 1), (128, 256, 6272, 2), (129, 256, 8192, 1), (129, 256, 8320, 2), (4, 256, 65536, 2),  # few tiles
+    (9800, 256, 8320, 1),                                       # more tiles than half of the SMs: nothing to split
+    (300, 384, 2048, 2), (300, 192, 2112, 2), (300, 256, 2112, 2),  # widths and K that the pairs do not take
+    (300, 384, 1984, 1)])
+def test_gemm_kernel_by_shape(M, N, K, nodes):
+    # a captured call is one kernel on CTA pairs or on single CTAs without a
+    # split, and split K clears its arrival counters before: very long sums of
+    # few tiles go there (on a pair 4 x 256 x 65536 takes 158 us, split 42)
+    cuda = ctypes.CDLL("libcuda.so.1")
+    A, Bw = torch.zeros((M, K), dtype=torch.bfloat16, device="cuda"), torch.zeros((N, K), dtype=torch.bfloat16, device="cuda")
+    out = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    f3dc.gemm(A, Bw, None, None, out, M, N, K, f3dc.EPI_BIAS)  # the workspace is allocated on first use
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
+    assert cuda.cuStreamBeginCapture_v2(ctypes.c_void_p(s.cuda_stream), 2) == 0  # relaxed
+    f3dc.gemm(A, Bw, None, None, out, M, N, K, f3dc.EPI_BIAS, stream=s.cuda_stream)
+    assert cuda.cuStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph)) == 0
+    assert cuda.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    assert cuda.cuGraphDestroy(graph) == 0
+    assert n.value == nodes
