@@ -41,8 +41,12 @@ def _tiny_step_clean():
     h.close()
 
 
-def test_split_k_wait_runs_out_and_is_reported():
-    M, N, K = 300, 1024, 4096  # 12 tiles on 152 SMs: K is split
+@pytest.mark.parametrize("N", [1024, 384])
+def test_split_k_wait_runs_out_and_is_reported(N):
+    # 12 or 9 tiles on 152 SMs: with the injection on, both split K.  After it
+    # N 1024 runs on CTA pairs, N 384 splits again: the counters that the
+    # timeout left raised are cleared.
+    M, K = 300, 4096
     A, Bw, bias = _gemm_inputs(M, N, K, 1)
     assert f3dc.gemm_status() == 0
     out = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")

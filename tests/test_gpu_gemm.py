@@ -15,9 +15,12 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [(1229, 1024, 1024), (4096, 3072, 1024), (1000, 4096, 1024), (1229, 1024, 4096), (100, 256, 128),
           (1, 64, 64), (257, 384, 128), (300, 128, 256)]
-# few row tiles: the kernel splits K over CTAs and reduces the partials in
-# split order (workspace + per-tile arrival counters)
-SPLIT_SHAPES = [(955, 1024, 1024), (300, 1024, 4096), (128, 256, 1024), (640, 3072, 1024), (413, 1024, 4096)]
+# few row tiles.  On CTA pairs (N a multiple of 256, K of 128): whole sums of K
+# 1024, sums in pieces of K 4096.  Otherwise, and beyond K 8192, single CTAs split
+# K and reduce the partials in split order (workspace + per-tile arrival counters):
+# tiles of 128, 64 and 256 columns, 3 to 16 splits.
+SPLIT_SHAPES = [(955, 1024, 1024), (300, 1024, 4096), (128, 256, 1024), (640, 3072, 1024), (413, 1024, 4096),
+                (300, 384, 4096), (413, 192, 2048), (128, 64, 4096), (1100, 640, 2112), (300, 256, 2112), (5, 512, 8448)]
 
 
 def _inputs(M, N, K, seed):
@@ -49,7 +52,7 @@ def test_gemm_bias(orc, M, N, K):
     assert np.all(np.abs(got - ref) <= 2.0 ** -7 * np.abs(ref) + 1e-3)
 
 
-@pytest.mark.parametrize("M,N,K", SHAPES[:4] + SPLIT_SHAPES[:2])
+@pytest.mark.parametrize("M,N,K", SHAPES[:4] + SPLIT_SHAPES[:2] + SPLIT_SHAPES[5:])
 def test_gemm_gelu(orc, M, N, K):
     A, Bw, bias, _, rows = _inputs(M, N, K, 7 + M)
     out = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
@@ -97,10 +100,10 @@ def test_gemm_no_bias_and_repeat_is_deterministic(orc):
     assert rel_l2(outs[0].float().cpu().numpy()[rows], ref) < 4e-3
 
 
-def test_gemm_split_k_repeat_is_deterministic(orc):
-    # the split partials are always summed in split order by whichever CTA
-    # arrives last, so repeated launches agree bit for bit
-    M, N, K = 300, 1024, 4096
+@pytest.mark.parametrize("M,N,K", [(300, 1024, 4096), (300, 384, 4096), (300, 256, 2112)])
+def test_gemm_split_k_repeat_is_deterministic(orc, M, N, K):
+    # pieces are summed in order, split partials in split order by whichever
+    # CTA arrives last, so repeated launches agree bit for bit
     A, Bw, bias, gate, rows = _inputs(M, N, K, 21)
     outs = []
     for _ in range(3):

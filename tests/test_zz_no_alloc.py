@@ -3,9 +3,9 @@
 allocation, loops that must not enter the driver's allocator).  Its split-K
 scratch is a fixed array inside libf3dc instead of an allocation, and it
 makes f3dc_gemm's launch decisions, so its output must equal f3dc_gemm's bit
-for bit -- here on two split calls in a row with different split counts (the
-second starts from whatever the first left in the shared array), on shapes
-that take the CTA-pair kernel, and once against the oracle.
+for bit -- here on split calls in a row with different split counts (each
+starts from whatever the one before left in the shared array), on shapes that
+take the CTA-pair kernel, and against the oracle.
 
 This file is collected last so that a run which stops at the first failure
 has already run every other test."""
@@ -22,8 +22,12 @@ pytestmark = pytest.mark.gpu
 def _split_count(M, N, K, sms):
     """The library's split-K rule for a standalone GEMM (host restatement):
     split only when whole 128-row tiles leave at least half of the grid idle
-    and K >= 2048, >= 4 K blocks of 64 per split, no empty split."""
+    and K >= 2048, >= 4 K blocks of 64 per split, no empty split; 1 for what
+    runs on CTA pairs (256-wide, K a multiple of 128 up to 8192, 6144 with one
+    row tile)."""
     bn = 256 if N % 256 == 0 else (128 if N % 128 == 0 else 64)
+    if bn == 256 and K % 128 == 0 and K <= (8192 if M > 128 else 6144):
+        return 1
     tiles = -(-M // 128) * (N // bn)
     grid = sms if 2 * tiles <= sms else min(tiles, sms)
     kb = K // 64
@@ -64,9 +68,10 @@ def _both(M, N, K, epi, seed):
 
 def test_noalloc_equals_gemm_on_two_split_calls_in_a_row(orc):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    cases = [(300, 1024, 4096, f3dc.EPI_RESID, 1), (200, 1024, 2048, f3dc.EPI_BIAS, 2)]
+    cases = [(300, 384, 4096, f3dc.EPI_RESID, 1), (200, 192, 2048, f3dc.EPI_BIAS, 2),
+             (1100, 640, 2112, f3dc.EPI_RESID, 3), (5, 512, 8448, f3dc.EPI_RESID, 4)]
     counts = [_split_count(M, N, K, sms) for M, N, K, _, _ in cases]
-    assert counts[0] > 1 and counts[1] > 1 and counts[0] != counts[1], counts
+    assert min(counts) > 1 and len(set(counts)) > 2 and counts[0] != counts[1], counts
     for (M, N, K, epi, seed) in cases:
         got, ref, (A, Bw, bias, gate, x0) = _both(M, N, K, epi, seed)
         np.testing.assert_array_equal(got, ref)
@@ -81,10 +86,11 @@ def test_noalloc_equals_gemm_on_two_split_calls_in_a_row(orc):
 
 
 def test_noalloc_equals_gemm_without_split():
-    # the CTA-pair kernel (256-wide tiles, K % 128 == 0, no split) and the
-    # single-CTA kernel for a 128-wide N
+    # the CTA-pair kernel (256-wide tiles, K % 128 == 0; the last two sum in
+    # pieces) and the single-CTA kernel for a 128-wide N
     for M, N, K, epi, seed in [(4096, 3072, 1024, f3dc.EPI_GELU, 3), (128, 256, 1024, f3dc.EPI_GELU, 4),
-                               (955, 1024, 1024, f3dc.EPI_BIAS, 5), (300, 384, 512, f3dc.EPI_RESID, 6)]:
+                               (955, 1024, 1024, f3dc.EPI_BIAS, 5), (300, 384, 512, f3dc.EPI_RESID, 6),
+                               (300, 1024, 4096, f3dc.EPI_RESID, 1), (200, 1024, 2048, f3dc.EPI_BIAS, 2)]:
         got, ref, _ = _both(M, N, K, epi, seed)
         np.testing.assert_array_equal(got, ref)
         assert rel_l2(got, ref) == 0.0
