@@ -1466,6 +1466,7 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
     cudaStream_t s = (cudaStream_t)stream;
     if (pair) {
         p.piece_kb = gemm_piece_kb(K, splits);
+        p.rows_first = gemm_rows_first(M, N, K);
         CK(launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s));
         return F3DC_OK;
     }

@@ -636,17 +636,18 @@ constexpr size_t kPairSmem = 1024 + (size_t)kPairStages * (kPairAStage + kPairBS
 // more operand bytes per product (its 256 rows of A are read for fewer
 // columns), so it only pays on clusters that would idle: 1229 x 4096 x 1024
 // (80 tiles on 76 clusters) 16.2 -> 12.7 us, 4096 x 4096 x 1024 27.7 -> 24.0.
-// Units run column-fastest: the weights (8 MB at most here) stay in L2 and each
-// row block of A is read from memory once, also when A is larger than L2
-// (25000 x 1024 x 4096: 177 us row-fastest, 130).
+// Units run column-fastest: the weights stay in L2 and each row block of A is read
+// from memory once, also when A is larger than L2 (25000 x 1024 x 4096: 177 us
+// row-fastest, 130).  With `rows_first` they run row-fastest (gemm_rows_first).
 struct PairUnits {
-    int n_tiles, full, sub, total;  // column tiles; full-width units; pieces of each other tile; units
-    float inv_n;
-    F3DC_DEV PairUnits(int pm_tiles, int N, int clusters, int rows)
+    int line, full, sub, total;  // tiles of a row (column); full-width units; pieces of each other tile; units
+    float inv_line;
+    bool rows_first;
+    F3DC_DEV PairUnits(int pm_tiles, int N, int clusters, int rows, bool rows_first_) : rows_first(rows_first_)
     {
-        n_tiles = N / 256;
-        inv_n = 1.0f / (float)n_tiles;
-        const int tiles = pm_tiles * n_tiles;
+        line = rows_first ? pm_tiles : N / 256;
+        inv_line = 1.0f / (float)line;
+        const int tiles = pm_tiles * (N / 256);
         full = tiles / clusters * clusters;
         const int rest = tiles - full;
         // a handful of rows is read by every cluster from the same few L2 lines:
@@ -665,24 +666,26 @@ struct PairUnits {
             piece = v & (sub - 1);
             bn = 256 >> log_sub;
         }
-        // tile / n_tiles: the quotient's distance to an integer is at least
-        // 0.5 / n_tiles, the rounding error below tile / n_tiles * 2^-22
-        m = (int)(((float)tile + 0.5f) * inv_n);
-        n0 = (tile - m * n_tiles) * 256 + piece * bn;
+        // tile / line: the quotient's distance to an integer is at least
+        // 0.5 / line, the rounding error below tile / line * 2^-22
+        const int q = (int)(((float)tile + 0.5f) * inv_line), r = tile - q * line;
+        m = rows_first ? r : q;
+        n0 = (rows_first ? q : r) * 256 + piece * bn;
     }
 };
 
 // kPieces: a unit's K is summed in pieces of at most p.piece_kb stages, each in an
 // accumulator of its own, added in order in fp32.  The tensor core truncates as it
-// accumulates, so the error of a sum grows with its length (of random signs, 4096:
-// 3.2e-6 relative, 1024: 1e-6, 256: 2.4e-7).  TMEM holds 512 / bn accumulators: the first takes the
+// accumulates, so the error of a sum grows with its length (random signs, relative:
+// 4096 4.4e-6, 1024 1.0e-6, 256 2.3e-7; positive products 1.4e-5, 2.2e-6, 3.8e-7).  TMEM holds 512 / bn accumulators: the first takes the
 // sum, and where there are more pieces than accumulators the others take turns,
 // the epilogue warps adding one while the next is computed.  A kernel of its own:
 // the steps' launches sum the whole K and start with a cold instruction cache.
 // Error (2-norm, positive products) and time of one sum of the whole K, of pieces,
-// and of the single-CTA kernel's split K: 1 x 1024 x 4096 9e-6 (four accumulators
-// without turns: 2.2e-6, 14.7 us), 16 pieces 3.8e-7, 20 us, split K 3.8e-7, 29.5 us;
-// 1229 x 1024 x 4096 four pieces 2.2e-6, 17.3 us, split K 3.0e-6, 30.8 us.
+// and of the single-CTA kernel's split K: 1 x 1024 x 4096 1.4e-5, 13.5 us (four
+// pieces 2.2e-6, 14.7 us), 16 pieces 3.8e-7, 20 us, split K 3.8e-7, 29.5 us;
+// 1229 x 1024 x 4096 1.4e-5, 16.5 us, four pieces 2.2e-6, 17.3 us, split K 3.0e-6,
+// 30.8 us.
 template <int EPI, bool kPieces>
 __global__ void __launch_bounds__(kPairThreads, 1)
     k_gemm_pair(const __grid_constant__ CUtensorMap tma, const __grid_constant__ GemmPairB tmb,
@@ -746,7 +749,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const int m_tiles = __shfl_sync(0xffffffffu, p.m_tiles_dev ? ld_plan(p.m_tiles_dev) : p.m_tiles, 0);
     const int kb_n = p.K / kPairBK;
     const int cl = blockIdx.x >> 1, ncl = gridDim.x >> 1;
-    const PairUnits U((m_tiles + 1) / 2, p.N, ncl, p.M);
+    const PairUnits U((m_tiles + 1) / 2, p.N, ncl, p.M, p.rows_first != 0);
     // In a step B is a weight: its part of the first stages is loaded before
     // the wait (the barrier's arrival and byte count follow with A's part), half
     // of what the first MMAs need: a cached step of 24 blocks at 1229 tokens

@@ -169,6 +169,7 @@ struct GemmParams {
     // CTA pairs: longest sum in one accumulator, in stages of 128 K (0: the whole
     // K), see gemm_piece_kb
     int piece_kb;
+    int rows_first;  // CTA pairs: order of the units, see gemm_rows_first
     // fault injection (tests of the failure path; 0 in normal use): the
     // split-K arrival wait expects split_extra arrivals beyond the splits
     // that exist, and gives up after split_wait_ns (0: kWaitLimitNs)
@@ -213,6 +214,14 @@ inline bool gemm_on_pairs(int M, int N, int K, int splits)
 {
     return N % 256 == 0 && K % 128 == 0 && (splits == 1 || K <= (M > kTileRows ? 8192 : 6144));
 }
+// Weights that do not stay in L2 (129 MB) next to what streams through it are read
+// again by every wave of column-fastest units; row-fastest ones read A again
+// instead, which is better where A is the smaller.  Column- / row-fastest, us:
+// 5000 x 8192 x 8192 (134 MB of weights, 82 of A) 401 / 374, 5000 x 8192 x 4096 (67
+// and 41 MB) 193 / 179, 1400 x 8192 x 4096 (67, 11) 66.3 / 64.0; 5000 x 4096 x 8192
+// (67, 82) 223 / 228, 25000 x 4096 x 8192 (67, 410) 955 / 1157.  At 50 MB of weights
+// (5000 x 6144 x 4096) the order made no difference beyond the runs' own.
+inline bool gemm_rows_first(int M, int N, int K) { return M < N && (int64_t)N * K * 2 > (int64_t)64000000; }
 // Where launch_gemm would split K, its partial sums are shorter, and so more precise,
 // than one sum of the whole K: the pairs then sum pieces no longer than one of its
 // `splits` (which has at least four blocks of 64).

@@ -142,6 +142,7 @@ extern "C" f3dc_status f3dc_gemm_noalloc(const void *A, const void *B, const voi
     cudaStream_t s = (cudaStream_t)stream;
     if (pair) {
         p.piece_kb = gemm_piece_kb(K, splits);
+        p.rows_first = gemm_rows_first(M, N, K);
         e = launch_gemm_pair(&ta, &tbp, p, epi, (m_tiles + 1) / 2 * (N / 64), s);
         if (e != cudaSuccess) return fail(F3DC_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
         return F3DC_OK;

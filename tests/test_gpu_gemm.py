@@ -209,3 +209,23 @@ def test_gemm_kernel_by_shape(M, N, K, nodes):
     assert cuda.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
     assert cuda.cuGraphDestroy(graph) == 0
     assert n.value == nodes
+
+
+@pytest.mark.parametrize("M", [1, 300, 2500])
+def test_gemm_rows_first(M):
+    # 67 MB of weights and fewer rows than columns: units run row-fastest.  1, 2
+    # and 10 row pairs of 32 column tiles on 76 clusters: narrow units, full units
+    # only, and full waves with a rest.
+    N, K = 8192, 4096
+    g = torch.Generator(device="cuda").manual_seed(M)
+    A = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    Bw = (torch.randn(N, K, generator=g, device="cuda") / K ** 0.5).bfloat16()
+    out = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    f3dc.gemm(A, Bw, None, None, out, M, N, K, f3dc.EPI_RESID)
+    y = A.double() @ Bw.double().T
+    # K / 16 steps, each truncating 2^-24 of the sum so far on average: at most
+    # half of them, with a sum that grows to its final size (4.4e-6 measured, with
+    # column-fastest units too)
+    assert ((out.double() - y).norm() / y.norm()).item() < K / 32 * 2.0 ** -24
+    assert (out.double() - y).abs().max().item() < 1e-4
+    assert f3dc.gemm_status() == 0
