@@ -164,3 +164,62 @@ def test_selection_where_the_radix_search_ends(orc, h16, case):
     qs = np.array([q], np.int32)
     idx, na, mask = _run(h16, hist, qs)
     _check(orc, hist, qs, idx, na, mask)
+
+
+def _norm(x):
+    s = np.zeros(x.shape[:-1], np.float32)
+    for c in range(x.shape[-1]):
+        s = s + x[..., c] * x[..., c]
+    return np.sqrt(s)
+
+
+def _vector_of_norm(target, g):
+    # bf16 channels whose fp32 norm is `target` to the bit: a greedy expansion of
+    # its square from a random first channel
+    def floor_bf16(x):
+        return (np.asarray(x, np.float32).view(np.uint32) & np.uint32(0xFFFF0000)).view(np.float32)
+
+    x = np.zeros((4000, 8), np.float32)
+    rest = np.full(4000, float(target) ** 2)
+    x[:, 0] = floor_bf16(target * g.uniform(0.3, 0.95, 4000))
+    for c in range(1, 5):
+        rest = rest - x[:, c - 1].astype(np.float64) ** 2
+        x[:, c] = floor_bf16(np.sqrt(np.maximum(rest, 0)))
+    return x[np.flatnonzero(_norm(x) == target)[0]]
+
+
+def test_selection_where_one_ulp_of_a_quotient_decides(orc):
+    # 510 tokens of an 8^3 grid whose norms lie within 300 neighbouring floats, so
+    # that a quotient norm / range off by one ulp changes which are cached for some
+    # of the 511 quotas; ranges next to a power of two, with all ones, and others.
+    # For two of the ranges the product with the reciprocal alone is that far off
+    # (the rest of the score is 0 there), which shows that the quotas can tell.
+    N, omega = 512, 0.7
+    quotas = np.arange(1, N, dtype=np.int32)
+    told = 0
+    h, _, _ = handle_for(_shape(8), max_batch=64)
+    for mant in (1, 2, 3, 2 ** 23 - 1, 2 ** 23 - 2, 2 ** 22 - 1, 2 ** 22, 0x2AAAAB):
+        g = np.random.default_rng(mant)
+        top = np.uint32(127 << 23 | mant).view(np.float32)
+        base = np.float32(0.37 + 0.6 * g.random()) * top
+        v1 = np.zeros((N, 8), np.float32)  # token N - 2 stays 0: the range is `top`
+        for i in range(N - 2):
+            v1[i] = _vector_of_norm((base.view(np.uint32) + np.uint32(g.integers(0, 300))).view(np.float32), g)
+        v1[N - 1] = _vector_of_norm(top, g)
+        v2 = v1.copy()
+        v2[0, 7] = -1.0  # A is 1 for this token and 0 for the others
+        perm = g.permutation(N)
+        b1, b2 = (synth.f32_to_bf16_bits(x[perm]) for x in (v1, v2))
+        score = orc.ssc_score(b1, b2, omega)
+        rough = np.where(perm == 0, score, (np.float32(1) - np.float32(omega)) * (_norm(v1[perm]) * (np.float32(1) / top)))
+        for q0 in range(0, len(quotas), 64):
+            qs = quotas[q0:q0 + 64]
+            hist = np.stack([b2 * 0, b2, b1])[:, None].repeat(len(qs), 1)
+            idx, na, mask = _run(h, hist, qs)
+            for b, c in enumerate(qs):
+                cached, aidx = orc.select(score, int(c))
+                np.testing.assert_array_equal(mask[b], cached, err_msg=f"range {mant:#x}, quota {c}")
+                np.testing.assert_array_equal(idx[b, :na[b]], aidx)
+                told += not np.array_equal(orc.select(rough.astype(np.float32), int(c))[0], cached)
+    assert told > 100
+    h.close()
