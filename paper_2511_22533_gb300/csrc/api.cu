@@ -475,8 +475,9 @@ cudaError_t run_gemm(f3dc_handle *h, const f3dc_handle::OperandA &ta, const f3dc
     p.err = h->dev_err;
     // 256-wide tiles run on CTA pairs.  At most one cluster per 128 columns: a
     // model whose launches are all small (8^3 grid, width 128) is bound by their
-    // latency, and its sample takes 1017 us with 16-CTA launches of fc1, 1036
-    // with 32 (64-column units)
+    // latency, and its sample takes 956 us with 16-CTA launches of fc1, 1007 with
+    // 32 (64-column units).  At width 1024 the two are the same: a step of 8 blocks
+    // with 60 to 2000 active tokens 724 to 1082 us with either, within 0.1 %.
     if (bn == 256) return launch_gemm_pair(&ta.pair, &tb.pair, p, epi, (h->max_tiles + 1) / 2 * (N / 128), s);
     const int tiles = h->max_tiles * (N / bn);
     const int grid = tiles < h->num_sms ? tiles : h->num_sms;

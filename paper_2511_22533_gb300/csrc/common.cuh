@@ -350,19 +350,9 @@ F3DC_DEV void mma_commit_elect(uint64_t *bar)
 
 // D (+)= A B^T over a CTA pair: A rows 0..127 from this CTA's shared memory
 // and rows 128..255 from the peer's, at the same offsets; B's N rows split the
-// same way; D rows 0..127 in this CTA's TMEM, 128..255 in the peer's.
-F3DC_DEV void mma_bf16_pair_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                  uint32_t accumulate)
-{
-    asm volatile(
-        "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
-        " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The eight pair MMAs of 128 K (two 64-K regions of each operand, a_half and
-// b_half apart in descriptor units; 16 K further is 2 units) under one election.
+// same way; D rows 0..127 in this CTA's TMEM, 128..255 in the peer's.  The eight
+// MMAs of 128 K (two 64-K regions of each operand, a_half and b_half apart in
+// descriptor units; 16 K further is 2 units) under one election.
 F3DC_DEV void mma_bf16_pair_128k(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint64_t a_half, uint64_t b_half,
                                  uint32_t idesc, uint32_t accumulate)
 {
@@ -587,9 +577,9 @@ F3DC_DEV float warp_sum(float v)
 // LayerNorm of one row held by a warp (Supp. Sec. F; eps 1e-6): lane l holds
 // the float4 groups q * 32 + l (q < NV) of the row's W = 128 NV values.  The
 // mean first, then the mean of squared deviations, each summed per lane in
-// q order and then across the warp; every kernel that normalises rows (the
-// LayerNorm kernel, the final layer, the fused LayerNorm of the residual
-// GEMM) uses these two helpers, so their outputs agree bit for bit.
+// q order and then across the warp; both kernels that normalise rows (the
+// LayerNorm kernel and the final layer) take them from here, so their outputs
+// agree bit for bit.
 template <int NV>
 F3DC_DEV void ln_row_stats(const float4 (&v)[NV], int W, float &mean, float &rstd)
 {

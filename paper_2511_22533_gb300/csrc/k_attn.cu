@@ -61,7 +61,7 @@ namespace f3dc {
 
 namespace {
 
-constexpr int kAttnThreads = 384;  // producer, MMA issuer, two idle warps, 2 x 4 softmax warps
+constexpr int kAttnThreads = 384;  // producer, two MMA issuers, an idle warp, 2 x 4 softmax warps
 constexpr int kKVStages = 4;
 // Registers per thread after the split.  The launch has 384 x 168 = 64512; a
 // softmax thread holds a whole score row of a key tile (128 floats).

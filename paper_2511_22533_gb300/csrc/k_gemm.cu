@@ -601,13 +601,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
 // ------------------------------------------------------------ CTA pair
 // cta_group::2 GEMM for 256-wide tiles.  A cluster of two CTAs computes a
-// 256 x 256 tile (a launch's last wave 256 x 128 or 256 x 64): each CTA loads its 128 rows of A
-// and its half of the tile's B rows into its own shared memory (128 K per stage), the even CTA
-// issues the 256-row MMAs for both, and each CTA's TMEM receives its own 128
-// rows of the accumulator, which its epilogue warps write out.  Per SM that
-// is 32 KB of operands per 512 MMA clocks instead of the 48 KB a 128 x 256
-// tile of one CTA needs, so the operand stream from L2 keeps up with the
-// tensor core.
+// 256 x 256 tile (in a launch's last wave also 256 x 128 or 256 x 64): each CTA
+// loads its 128 rows of A and its half of the tile's B rows into its own shared
+// memory (128 K per stage), the even CTA issues the 256-row MMAs for both, and
+// each CTA's TMEM receives its own 128 rows of the accumulator, which its
+// epilogue warps write out.  Per SM a full-width unit takes 32 KB of operands per
+// 512 MMA clocks instead of the 48 KB of a 128 x 256 tile of one CTA, so the
+// operand stream from L2 keeps up with the tensor core (128 columns: 24 KB per
+// 256 clocks, 64: 20 KB per 128).
 //   full[s]  (even CTA): both CTAs' TMA bytes of stage s (the even CTA's
 //            producer posts the expected count)
 //   empty[s] (both):     stage s consumed (multicast MMA commit)
@@ -631,8 +632,9 @@ constexpr size_t kPairSmem = 1024 + (size_t)kPairStages * (kPairAStage + kPairBS
 
 // Work units of a launch whose row count is only known on the device: full
 // waves of 256-wide tiles, and the tiles left for the last wave cut into 2 or 4
-// units of 128 or 64 columns when that many clusters are free for them (a
-// launch of less than half a wave is all last wave).  A narrower unit costs
+// units of 128 or 64 columns when that many clusters are free for all of them (a
+// launch of less than half a wave is all last wave; 39 tiles left for 76 clusters
+// stay whole).  A narrower unit costs
 // more operand bytes per product (its 256 rows of A are read for fewer
 // columns), so it only pays on clusters that would idle: 1229 x 4096 x 1024
 // (80 tiles on 76 clusters) 16.2 -> 12.7 us, 4096 x 4096 x 1024 27.7 -> 24.0.
@@ -651,7 +653,10 @@ struct PairUnits {
         full = tiles / clusters * clusters;
         const int rest = tiles - full;
         // a handful of rows is read by every cluster from the same few L2 lines:
-        // more clusters wait longer (1 x 4096 x 1024: 10.5 us on 64 clusters, 8.9 on 32)
+        // more clusters wait longer.  64 / 32 clusters, us: 1 x 4096 x 1024 10.4 / 8.7,
+        // 16 rows 8.7 / 6.8, 63 rows 9.5 / 8.2, 64 rows 6.2; 48 / 24 clusters: 16 x 3072 x
+        // 1024 7.8 / 6.4; 16 / 8: 1 x 1024 x 1024 6.6 / 6.0, but 16 rows 5.3 / 6.0.  (A step
+        // passes its capacity: all rows of a tile are loaded there.)
         sub = 4 * rest <= clusters && rows >= 64 ? 4 : (2 * rest <= clusters ? 2 : 1);
         total = full + rest * sub;
     }
