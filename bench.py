@@ -51,7 +51,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 GEMM_TRAFFIC = {"dram_bytes_per_launch": 68.9e6 / 6, "algorithmic_bytes_per_launch": 67.1e6 / 6,
                 "shape": "QKV, attention out, cross Q, cross out, fc1, fc2 at 1229 active rows, width 1024",
                 "profile": "profiles/k_gemm_pair_cached_step_1229rows.md",
-                "k_gemm_cu_sha256": "e864edcda82fbe64c11ba4eddb23777ac3186614f63be50dc7fb04ba6053839b"}
+                "k_gemm_cu_sha256": "ba9780e73c9705b126ee04454ed7334824672ec57ee7440dbdc80b1ef22dc02a"}
 
 
 def parse():

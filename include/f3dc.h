@@ -343,7 +343,7 @@ f3dc_status f3dc_gemm(const void *A, const void *B, const void *bias, const floa
  * latency-critical loops must not enter the driver's allocator; f3dc_gemm,
  * which allocates its split-K workspace on first use per device, serves none
  * of them.  This call makes f3dc_gemm's launch decisions (the CTA-pair kernel
- * where N and K allow, otherwise the single-CTA kernel with the same split
+ * for the same shapes, otherwise the single-CTA kernel with the same split
  * rule and summation order), so its output equals f3dc_gemm's
  * bit for bit, with the same arguments and errors; but it takes the split-K
  * workspace from a fixed 20 MiB array (plus 4 KiB of counters) compiled into

@@ -40,9 +40,9 @@
 // no maximum and has no branch on the data.
 // What bounds it: the softmax warps.  Per key tile of 128 x 128 scores an SM's
 // exponent unit needs 512 clocks (32 per clock) and the tensor core 512; the
-// kernel takes ~950 (4096 x 4096 x 16 heads, dh 64: 63.9 us = 1075 TFLOP/s;
-// before -- one issuer warp, a maximum of every half tile, ~1250 clocks --
-// 79.1 us; 1229 x 1374: 17.6 -> 15.9 us).  A softmax warp alone needs ~730
+// kernel takes ~950 (4096 x 4096 x 16 heads, dh 64, back to back: 63.4 us = 1083
+// TFLOP/s; before -- one issuer warp, a maximum of every half tile, ~1250 clocks
+// -- 79.1 us; 1229 x 1374: 17.6 -> 15.5 us).  A softmax warp alone needs ~730
 // clocks per tile (load, exponents, store), and the two of an SM sub-partition
 // mostly compete for the exponent unit at the same time.  Measured slower: 16
 // softmax warps with half a row each (73 us: the waits' instructions double),
@@ -83,7 +83,13 @@ struct AttnCfg {
 };
 
 // A CTA's items run in windows of this many: a first pass over the window, then a
-// second one over the items in which a row asked for it (a bit for each).
+// second one over the items in which a row asked for it (a bit for each).  Against
+// a second pass over all of a CTA's items that stores all their rows, so that one
+// sample's data changes another's bits, this costs code and registers: 4096 x 4096
+// 64.7 -> 65.3 us (L2 flushed), 1229 x 1374 15.7 -> 15.9, a sample of the 8^3 model
+// 947 -> 957.  Measured slower still: the range from the first to the last such item
+// instead of bits (66.8 us, 16.6, 962), item data kept in shared memory over the key
+// loop (65.8, 16.0, 962).
 constexpr int kWindow = 32;
 
 struct Item {
