@@ -194,27 +194,31 @@ def _bits(t):
     return t.view(torch.int16).cpu().numpy()
 
 
-@pytest.mark.parametrize("nq,nk,H,dh", [(2700, 900, 16, 64), (4096, 700, 16, 64), (4096, 700, 16, 32)])
+@pytest.mark.parametrize("nq,nk,H,dh", [(2700, 900, 16, 64), (4096, 700, 16, 64), (4096, 700, 16, 32),
+                                        (20000, 640, 64, 32)])
 @pytest.mark.parametrize("which", ["all", "one"])
 def test_attention_second_pass_over_several_items(orc, nq, nk, H, dh, which):
     # 176 and 256 (pair, head) items on 152 SMs: CTAs with one item and CTAs
     # with two, whose second pass starts at other K/V stages, Q buffers and
-    # barrier phases than the first did.  "all": every row's scores rise by
-    # 2^90 after the first key tile, so every item runs twice.  "one": a single
-    # row of one head does, in the second item of its CTA (152 + 3), and only
-    # that item does.  Written over the queries the result is the same.
+    # barrier phases than the first did; and 5056 items: 33 or 34 a CTA, more
+    # than a window of 32.  "all": every row's scores rise by 2^90 after the
+    # first key tile (and no ragged last tile raises the reference), so every
+    # item runs twice.  "one": a single row of one head does, in its CTA's last
+    # item, and only that item does.  Written over the queries the result is
+    # the same.
     g = np.random.default_rng(nq + nk + dh)
     W = H * dh
     u = np.where(g.random((H, dh)) < 0.5, -1.0, 1.0)
     unit = 1.0 / (np.sqrt(dh) * np.log2(np.e))
     a = np.zeros(nk)
     a[200:300] = 90.0 * unit
-    a[nk - 30:] = 80.0 * unit
+    a[400:450] = 101.0 * unit
     k = (np.einsum("j,hd->jhd", a, u) + 0.02 * g.standard_normal((nk, H, dh))).reshape(nk, W)
     v = g.standard_normal((nk, W))
     # strength 0.01: scores up to 0.9
     c = np.full((nq, H), 1.0 if which == "all" else 0.01)
-    item = 152 + 3
+    items = (nq + 255) // 256 * H
+    item = (items - 1) // 152 * 152 + 3
     row, head = 256 * (item // H) + 5, item % H
     c[row, head] = 1.0
     q = np.einsum("rh,hd->rhd", c, u).reshape(nq, W)

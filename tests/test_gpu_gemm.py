@@ -154,12 +154,14 @@ def _split_length(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K", [(1, 1024, 4096), (64, 1024, 4096), (128, 1024, 2048), (77, 512, 5120),
-                                   (300, 1024, 4096), (500, 2048, 2176), (384, 6400, 2048), (129, 256, 8192)])
+                                   (300, 1024, 4096), (500, 2048, 2176), (384, 6400, 2048), (129, 256, 8192),
+                                   (100, 12800, 4096)])
 @pytest.mark.parametrize("epi", [f3dc.EPI_BIAS, f3dc.EPI_GELU, f3dc.EPI_RESID])
 def test_gemm_long_sums_in_pieces(M, N, K, epi):
     # few tiles and a long K: sums in pieces no longer than split K's, in units of
     # 64, 128 and 256 columns, with fewer and more pieces than TMEM holds
-    # accumulators (2 to 16), and a last piece that is shorter.  Positive
+    # accumulators (2 to 16; the last shape three in two), and a last piece that
+    # is shorter.  Positive
     # products, so that truncation adds up: a step of 16 K loses 2^-24 of the sum
     # so far on average (up to 2^-23), a piece of L (L / 32) 2^-24 = 1.9e-9 L of
     # itself, the fp32 sum of the pieces about 1e-7.  A bias close to -sum shows
